@@ -2,13 +2,18 @@
 // 4.2, 4.3): median binning of consecutive frames, fake companion injection
 // into raw frames, aperture photometry of the reduced image.
 //
-//  * bin_median_kernel<W>: one thread per (group, pixel); the group's B <= W
-//    values are loaded (coalesced along the pixels, all loads in flight),
-//    turned into total-order keys padded with the largest key, sorted by a
-//    bitonic network in registers (all indices compile-time) and the median
-//    taken by the collapse rule.  HBM-bound: T x n^2 x 4 B read, ceil(T/B) x
-//    n^2 x 4 B written.  Groups of more than 64 frames go to the median
-//    collapse kernel, one launch per group.
+//  * bin_median_kernel<W, V>: one thread per group and V pixels; the group's
+//    B <= W values are loaded (coalesced along the pixels, all loads in
+//    flight) and the two middle ones of W slots taken by an odd-even merge
+//    network pruned to them, in registers (all indices compile-time).
+//    HBM-bound: T x n^2 x 4 B read, ceil(T/B) x n^2 x 4 B written.
+//    1000 frames of 512 x 512 by 10: 0.167 ms = 6.9 TB/s, the copy rate
+//    (0.60 with a 16-key bitonic sort of total-order keys).  Loading two
+//    pixels per thread with every load ahead of the first comparison, in a
+//    branch of its own for full bins, is what brings it there: with the
+//    slot tests between the loads it ran at 4.7 TB/s.
+//    Groups of more than 64 frames go to the median collapse kernel, one
+//    launch per group.
 //  * inject_kernel: one block per frame; companions in turn (a barrier
 //    between them, so overlapping windows never race), each over its window
 //    of (2 half + 1)^2 pixels; positions and windows come from the FP64 host
@@ -20,67 +25,71 @@
 #include <stdint.h>
 
 #include "graphic_internal.h"
+#include "select_common.cuh"
 
 namespace graphic {
 namespace {
 
 constexpr int BIN_THREADS = 128;
 
-__device__ __forceinline__ uint32_t bkey(float x) {
-  const uint32_t b = __float_as_uint(x);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-__device__ __forceinline__ float bval(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-
-template <int W>
+// V pixels per thread (V = 2: 8-byte loads) and W value slots per pixel, W
+// even and at least the group's m values.  The W - m free slots are padded
+// with -inf and +inf so that the middle values of the m sit in the middle of
+// the W: (W - m) / 2 of them, rounded down, below (an odd m leaves one more
+// above).  All loads are issued before the first comparison.
+template <int W, int V>
 __global__ void __launch_bounds__(BIN_THREADS) bin_median_kernel(const float *__restrict__ in, float *__restrict__ out,
                                                                  long long T, long long nn, int B,
-                                                                 long long blocks_per_group, int *status) {
+                                                                 unsigned blocks_per_group, int *status) {
   const long long g = blockIdx.x / blocks_per_group;
-  const long long p = (blockIdx.x - g * blocks_per_group) * BIN_THREADS + threadIdx.x;
+  const long long p = ((long long)(blockIdx.x % blocks_per_group) * BIN_THREADS + threadIdx.x) * V;
   if (p >= nn) return;
   const long long f0 = g * B;
   const int m = (int)((T - f0) < B ? (T - f0) : B);
   const float *src = in + f0 * nn + p;
-  uint32_t k[W];
-  bool bad = false;
-#pragma unroll
-  for (int i = 0; i < W; i++) {
-    if (i < m) {
-      const float v = __ldcs(src + (long long)i * nn);
-      bad |= !(fabsf(v) <= 3.402823466e38f);
-      k[i] = bkey(v);
+  float v[V][W];
+  float acc = 0.f;   // 0 while every value is finite: v * 0 is NaN for NaN and infinities
+  auto load = [&](int i) {
+    if constexpr (V == 2) {
+      const float2 x = __ldcs(reinterpret_cast<const float2 *>(src + (long long)i * nn));
+      v[0][i] = x.x;
+      v[V - 1][i] = x.y;
     } else {
-      k[i] = 0xffffffffu;
+      v[0][i] = __ldcs(src + (long long)i * nn);
+    }
+  };
+  if (m == W) {   // a full bin of the network's own width: no slot to test
+#pragma unroll
+    for (int i = 0; i < W; i++) load(i);
+#pragma unroll
+    for (int i = 0; i < W; i++)
+#pragma unroll
+      for (int u = 0; u < V; u++) acc = fmaf(v[u][i], 0.f, acc);
+  } else {
+#pragma unroll
+    for (int i = 0; i < W; i++) {
+      if (i < m) {
+        load(i);
+#pragma unroll
+        for (int u = 0; u < V; u++) acc = fmaf(v[u][i], 0.f, acc);
+      } else {
+#pragma unroll
+        for (int u = 0; u < V; u++) v[u][i] = ((i - m) & 1) ? -INFINITY : INFINITY;
+      }
     }
   }
-  if (bad) atomicOr(status, STATUS_NONFINITE);
+  if (!(acc == 0.f)) atomicOr(status, STATUS_NONFINITE);
+  float med[V];
 #pragma unroll
-  for (int s = 2; s <= W; s <<= 1)
-#pragma unroll
-    for (int j = s >> 1; j > 0; j >>= 1)
-#pragma unroll
-      for (int i = 0; i < W; i++) {
-        const int l = i ^ j;
-        if (l > i) {
-          const uint32_t a = k[i], b = k[l];
-          const bool up = (i & s) == 0;
-          k[i] = up ? min(a, b) : max(a, b);
-          k[l] = up ? max(a, b) : min(a, b);
-        }
-      }
-  const int ilo = (m - 1) >> 1, ihi = m >> 1;
-  uint32_t lo = 0, hi = 0;
-#pragma unroll
-  for (int i = 0; i < W; i++) {
-    if (i == ilo) lo = k[i];
-    if (i == ihi) hi = k[i];
+  for (int u = 0; u < V; u++) {
+    middle_pair<W>(v[u]);
+    const float lo = v[u][W / 2 - 1], hi = v[u][W / 2];
+    med[u] = (m & 1) ? lo : (lo + hi) * 0.5f;
   }
-  const float a = bval(lo);
-  out[g * nn + p] = (m & 1) ? a : (a + bval(hi)) * 0.5f;
+  if constexpr (V == 2)
+    *reinterpret_cast<float2 *>(out + g * nn + p) = make_float2(med[0], med[V - 1]);
+  else
+    out[g * nn + p] = med[0];
 }
 
 __global__ void inject_kernel(float *cube, long long T, int n, int n_comp, const double *__restrict__ pos,
@@ -136,13 +145,14 @@ __global__ void aperture_kernel(const float *__restrict__ img, int n, const doub
   }
 }
 
-template <int W>
+template <int W, int V>
 cudaError_t bin_launch(const float *in, float *out, long long T, long long nn, int B, int *status,
                        cudaStream_t st) {
   const long long G = (T + B - 1) / B;
-  const long long bpg = (nn + BIN_THREADS - 1) / BIN_THREADS;
-  if (G * bpg > 0x7fffffffLL) return cudaErrorInvalidConfiguration;   // one block per (bin, 128 pixels)
-  bin_median_kernel<W><<<(unsigned)(G * bpg), BIN_THREADS, 0, st>>>(in, out, T, nn, B, bpg, status);
+  const long long bpg = (nn + BIN_THREADS * V - 1) / (BIN_THREADS * V);
+  // one block per (bin, 128 or 256 pixels); the limit of the one-pixel form holds for both
+  if (G * ((nn + BIN_THREADS - 1) / BIN_THREADS) > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  bin_median_kernel<W, V><<<(unsigned)(G * bpg), BIN_THREADS, 0, st>>>(in, out, T, nn, B, (unsigned)bpg, status);
   return cudaGetLastError();
 }
 
@@ -155,13 +165,24 @@ cudaError_t launch_bin_median(const float *in, float *out, long long T, int n, i
   const long long nn = (long long)n * n;
   const long long G = (T + B - 1) / B;
   cudaError_t e;
-  if (B <= 16) {
-    e = bin_launch<16>(in, out, T, nn, B, status, st);
-  } else if (B <= 32) {
-    e = bin_launch<32>(in, out, T, nn, B, status, st);
-  } else if (B <= 64) {
-    e = bin_launch<64>(in, out, T, nn, B, status, st);
-  } else {
+  // the narrowest network that holds a bin (the comparators grow faster than
+  // W); two pixels per thread (8-byte loads) up to 32 values: 1000 frames of
+  // 512 x 512 in 165 us against 195 for B = 10, 185 / 194 for 32; from 40 on
+  // their registers cost more (B = 50: 240 us with one pixel, 260 with two)
+  if (B <= 2) e = bin_launch<2, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 4) e = bin_launch<4, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 6) e = bin_launch<6, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 8) e = bin_launch<8, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 10) e = bin_launch<10, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 12) e = bin_launch<12, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 16) e = bin_launch<16, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 20) e = bin_launch<20, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 24) e = bin_launch<24, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 32) e = bin_launch<32, 2>(in, out, T, nn, B, status, st);
+  else if (B <= 40) e = bin_launch<40, 1>(in, out, T, nn, B, status, st);
+  else if (B <= 50) e = bin_launch<50, 1>(in, out, T, nn, B, status, st);
+  else if (B <= 64) e = bin_launch<64, 1>(in, out, T, nn, B, status, st);
+  else {
     for (long long g = 0; g < G; g++) {
       CollapseArgs a{};
       a.in = in + g * B * nn;

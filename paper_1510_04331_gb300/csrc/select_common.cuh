@@ -39,6 +39,32 @@ __device__ __forceinline__ void cp_async_wait_group() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// The two middle order statistics of W values (W even) held in registers:
+// on return v[W/2 - 1] and v[W/2] are the ones a full sort would leave
+// there, the other slots are undefined.  Batcher's odd-even merge exchange
+// (Knuth, The Art of Computer Programming 3, 5.2.2, algorithm M); every
+// index is a compile-time constant, so the compiler drops the comparators
+// that no path leads from to the two results (W = 10: 31 comparators before
+// that, against 80 of a 16-key bitonic sort).  fminf / fmaxf order -0 below
+// +0 (PTX min / max), so equal-looking zeros come out in the total order.
+template <int W, int P, int K>
+__device__ __forceinline__ void merge_exchange(float (&v)[W]) {
+  constexpr int FIRST = (K == P) ? 0 : K;
+#pragma unroll
+  for (int x = FIRST; x < W - K; x++)
+    if ((((x - FIRST) / K) & 1) == 0 && x / (2 * P) == (x + K) / (2 * P)) {
+      const float a = v[x], b = v[x + K];
+      v[x] = fminf(a, b);
+      v[x + K] = fmaxf(a, b);
+    }
+  if constexpr (K > 1) merge_exchange<W, P, K / 2>(v);
+  else if constexpr (2 * P < W) merge_exchange<W, 2 * P, 2 * P>(v);
+}
+template <int W>
+__device__ __forceinline__ void middle_pair(float (&v)[W]) {
+  merge_exchange<W, 1, 1>(v);
+}
+
 // Position of the (r+1)-th set bit of x (r = 0 for the lowest), r < popc(x):
 // bisection on the popcounts of the low 16, 8, 4, 2 and 1 bits.
 __device__ __forceinline__ int nth_set(uint32_t x, int r) {
