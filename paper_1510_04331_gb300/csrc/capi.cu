@@ -37,7 +37,7 @@ struct graphic_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   int *d_status = nullptr;
-  int *h_status = nullptr;          // pinned
+  int *h_status = nullptr;          // pinned: the status word, then 8 bytes of results read back by a call
   char *d_plan = nullptr;
   size_t d_plan_bytes = 0;
   char *h_plan = nullptr;           // pinned staging
@@ -1339,7 +1339,7 @@ int graphic_create(graphic_ctx **out, int device) {
     return fail(GRAPHIC_ERR_CUDA, "twiddle table upload failed");
   }
   e = cudaMalloc(&c->d_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost(&c->h_status, sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost(&c->h_status, 4 * sizeof(int));
   if (e != cudaSuccess) {
     graphic_destroy(c);
     return cuda_fail(e, "context allocation");
@@ -1758,10 +1758,13 @@ int graphic_sky_median(graphic_ctx *c, const float *in, int64_t T, int32_t n, co
   if (!std::isfinite(mask_r) || mask_r < 0) return fail(GRAPHIC_ERR_INVALID_ARG, "mask_r must be finite, >= 0");
   DeviceGuard g(c->device);
   PlanBuilder pb;
-  size_t o_mx = 0, o_my = 0;
+  size_t o_mx = 0, o_my = 0, o_mf = 0;
   if (mask_x) {
     o_mx = pb.add(mask_x, T * sizeof(double));
     o_my = pb.add(mask_y, T * sizeof(double));
+    std::vector<float4> mf((size_t)T);
+    for (int64_t t = 0; t < T; t++) mf[t] = sky_mask_filter(mask_x[t], mask_y[t], mask_r, n);
+    o_mf = pb.add(mf.data(), T * sizeof(float4));
   }
   if ((rc = begin_call(c))) return rc;
   if ((rc = upload_plan(c, pb))) return rc;
@@ -1774,6 +1777,7 @@ int graphic_sky_median(graphic_ctx *c, const float *in, int64_t T, int32_t n, co
   a.mask_x = mask_x ? at<double>(c, o_mx) : nullptr;
   a.mask_y = mask_x ? at<double>(c, o_my) : nullptr;
   a.mask_r2 = mask_r * mask_r;
+  a.maskf = mask_x ? at<float4>(c, o_mf) : nullptr;
   prof_begin(c, GRAPHIC_K_COLLAPSE);
   cudaError_t e = launch_sky_median(a, c->stream);
   prof_end(c);
@@ -1805,91 +1809,19 @@ int graphic_sky_subtract(graphic_ctx *c, const float *in, float *out, int64_t T,
   return end_call(c);
 }
 
-namespace {
-
-// host value of a total-order key
-float key_value(uint32_t key) {
-  const uint32_t b = (key & 0x80000000u) ? (key & 0x7fffffffu) : ~key;
-  float f;
-  memcpy(&f, &b, sizeof f);
-  return f;
-}
-
-// Key of the k-th smallest (0-based) of n_vals device floats: four radix
-// passes, each a device histogram read back by the host.
-int select_key(graphic_ctx *c, const float *v, long long n_vals, unsigned long long k, unsigned int *d_hist,
-               uint32_t *key) {
-  uint32_t prefix = 0, pmask = 0;
-  unsigned long long krem = k;
-  std::vector<unsigned int> h(256);
-  for (int pass = 0; pass < 4; pass++) {
-    const int shift = 24 - 8 * pass;
-    cudaError_t e = launch_key_histogram(v, n_vals, prefix, pmask, shift, d_hist, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d_hist, 256 * sizeof(unsigned int), cudaMemcpyDeviceToHost,
-                                              c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "frame median");
-    unsigned long long cum = 0;
-    int d = 255;
-    for (int b = 0; b < 256; b++) {
-      if (cum + h[b] > krem) {
-        d = b;
-        break;
-      }
-      cum += h[b];
-    }
-    krem -= cum;
-    prefix |= (uint32_t)d << shift;
-    pmask |= 0xffu << shift;
-  }
-  *key = prefix;
-  return GRAPHIC_OK;
-}
-
-}  // namespace
-
 int graphic_bad_pixel_map(graphic_ctx *c, const float *ref, int32_t n, double C, uint8_t *map) {
   if (!c) return fail(GRAPHIC_ERR_INVALID_ARG, "null ctx");
   if (!ref || !map || n < 1) return fail(GRAPHIC_ERR_INVALID_ARG, "null buffer or n < 1");
   if (!std::isfinite(C) || C < 0) return fail(GRAPHIC_ERR_INVALID_ARG, "C must be finite, >= 0");
   DeviceGuard g(c->device);
-  const long long N = (long long)n * n;
   int rc;
-  if ((rc = ensure((void **)&c->d_prep, &c->prep_bytes, 4096, false))) return rc;
-  unsigned int *d_hist = reinterpret_cast<unsigned int *>(c->d_prep);          // 1 KB
-  double *d_sums = reinterpret_cast<double *>(c->d_prep + 1024);              // 2 doubles
-  double *d_mean = d_sums + 2;
-  double *d_thresh = d_sums + 3;
-  float *d_med = reinterpret_cast<float *>(c->d_prep + 1024 + 64);
-  double sums[2] = {0, 0};
-  CK(cudaMemsetAsync(d_sums, 0, 2 * sizeof(double), c->stream));
-  cudaError_t e = launch_frame_sums(ref, N, nullptr, d_sums, c->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "frame sums");
-  CK(cudaMemcpyAsync(sums, d_sums, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  if ((rc = ensure((void **)&c->d_prep, &c->prep_bytes, std::max<size_t>(4096, bad_map_bytes()), false))) return rc;
+  cudaError_t e = launch_bad_map(ref, (long long)n * n, C, map, c->d_prep, c->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "bad pixel map kernels");
+  volatile double *sum = reinterpret_cast<volatile double *>(c->h_status + 2);
+  CK(cudaMemcpyAsync(c->h_status + 2, c->d_prep, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  if (!std::isfinite(sums[0])) return fail(GRAPHIC_ERR_NONFINITE, "non-finite value in the reference frame");
-  const double mean = sums[0] / (double)N;
-  CK(cudaMemcpyAsync(d_mean, &mean, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  e = launch_frame_sums(ref, N, d_mean, d_sums, c->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "frame sums");
-  CK(cudaMemcpyAsync(sums, d_sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  const double sigma = sqrt(sums[1] / (double)N);
-  uint32_t klo, khi;
-  if ((rc = select_key(c, ref, N, (unsigned long long)((N - 1) / 2), d_hist, &klo))) return rc;
-  float med = key_value(klo);
-  if ((N & 1) == 0) {
-    if ((rc = select_key(c, ref, N, (unsigned long long)(N / 2), d_hist, &khi))) return rc;
-    const float hi = key_value(khi);
-    volatile float s = med + hi;   // FP32 sum, then the halving, as the device medians
-    med = s * 0.5f;
-  }
-  const double thresh = C * sigma;
-  CK(cudaMemcpyAsync(d_med, &med, sizeof(float), cudaMemcpyHostToDevice, c->stream));
-  CK(cudaMemcpyAsync(d_thresh, &thresh, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  e = launch_bad_map(ref, N, d_med, d_thresh, map, c->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "bad pixel map kernel");
-  CK(cudaStreamSynchronize(c->stream));
+  if (!std::isfinite(*sum)) return fail(GRAPHIC_ERR_NONFINITE, "non-finite value in the reference frame");
   return GRAPHIC_OK;
 }
 
@@ -1900,34 +1832,37 @@ int graphic_bad_pixel_fix(graphic_ctx *c, float *cube, int64_t T, int32_t n, con
   DeviceGuard g(c->device);
   const size_t bytes = (size_t)T * n * n * sizeof(float);
   int rc;
-  if ((rc = ensure((void **)&c->d_prep, &c->prep_bytes, 4096, false))) return rc;
+  if ((rc = ensure((void **)&c->d_prep, &c->prep_bytes, 4096 + fix_count_words(T) * sizeof(uint32_t), false))) return rc;
   if ((rc = ensure((void **)&c->d_scratch, &c->scratch_bytes, bytes, false))) return rc;
-  unsigned long long *d_cnt = reinterpret_cast<unsigned long long *>(c->d_prep + 2048);   // [3]
-  unsigned long long cnt[3] = {0, 0, 0};
-  CK(cudaMemsetAsync(d_cnt, 0, 3 * sizeof(unsigned long long), c->stream));
-  cudaError_t e = launch_bad_mark(cube, T, n, map, d_cnt, c->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "bad pixel marking kernel");
-  CK(cudaMemcpyAsync(cnt, d_cnt, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+  uint32_t *d_counts = reinterpret_cast<uint32_t *>(c->d_prep + 4096);
+  cudaError_t e = launch_bad_fill(cube, T, n, map, reinterpret_cast<uint32_t *>(c->d_scratch), d_counts, c->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "bad pixel correction kernels");
+  CK(cudaMemcpyAsync(c->h_status + 2, d_counts, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  unsigned long long left = cnt[0];
-  float *src = cube, *dst = c->d_scratch;
-  bool hopeless = false;
-  for (int pass = 0; left > 0 && pass <= 2 * n; pass++) {
-    CK(cudaMemsetAsync(d_cnt + 1, 0, 2 * sizeof(unsigned long long), c->stream));
-    e = launch_bad_pass(src, dst, T, n, d_cnt + 1, c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "bad pixel pass kernel");
-    CK(cudaMemcpyAsync(cnt + 1, d_cnt + 1, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    std::swap(src, dst);
-    if (cnt[2] == 0) {
-      hopeless = true;
-      break;
+  const uint32_t counts[2] = {(uint32_t)c->h_status[2], (uint32_t)c->h_status[3]};
+  bool hopeless = counts[1] > 0;
+  if (counts[0] > 0) {
+    // frames with more pixels to fill than a list holds: dense passes
+    // between the cube and the scratch, over every frame (the others hold no
+    // NaN any more)
+    unsigned long long *d_cnt = reinterpret_cast<unsigned long long *>(c->d_prep + 2048);   // [2]
+    unsigned long long cnt[2] = {1, 1};   // NaN left, filled
+    float *src = cube, *dst = c->d_scratch;
+    for (int pass = 0; cnt[0] > 0 && cnt[1] > 0 && pass <= 2 * n; pass++) {
+      CK(cudaMemsetAsync(d_cnt, 0, sizeof(cnt), c->stream));
+      e = launch_bad_pass(src, dst, T, n, d_cnt, c->stream);
+      if (e != cudaSuccess) return cuda_fail(e, "bad pixel pass kernel");
+      CK(cudaMemcpyAsync(cnt, d_cnt, sizeof(cnt), cudaMemcpyDeviceToHost, c->stream));
+      CK(cudaStreamSynchronize(c->stream));
+      std::swap(src, dst);
     }
-    left = cnt[1];
+    hopeless |= cnt[0] > 0;
+    if (src != cube) {
+      CK(cudaMemcpyAsync(cube, src, bytes, cudaMemcpyDeviceToDevice, c->stream));
+      CK(cudaStreamSynchronize(c->stream));
+    }
   }
-  if (src != cube) CK(cudaMemcpyAsync(cube, src, bytes, cudaMemcpyDeviceToDevice, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  if (hopeless || left > 0) return fail(GRAPHIC_ERR_NONFINITE, "a frame has no finite pixel left to fill from");
+  if (hopeless) return fail(GRAPHIC_ERR_NONFINITE, "a frame has no finite pixel left to fill from");
   return GRAPHIC_OK;
 }
 

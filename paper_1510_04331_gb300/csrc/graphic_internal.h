@@ -215,24 +215,34 @@ struct CollapseArgs {
   const double *mask_x;  // [T] device, may be null (no mask)
   const double *mask_y;
   double mask_r2;
+  const float4 *maskf;   // [T] device: (mask_x, mask_y, tolerance scale, row reach) in FP32 for
+                         // mask_covers (sky_mask_filter); null with mask_x null
 };
+// The FP32 filter of a star mask for frames of side n (CollapseArgs::maskf):
+// rows further than .w from .y are clear of it.
+float4 sky_mask_filter(double mask_x, double mask_y, double mask_r, int n);
 cudaError_t launch_collapse(const CollapseArgs &a, cudaStream_t st);
 cudaError_t launch_sky_median(const CollapseArgs &a, cudaStream_t st);
 
 // prep.cu: image-quality pre-processing (Sect. 3.2)
 cudaError_t launch_sky_subtract(const float *in, float *out, long long T, int n, const float *skies,
                                 const int *sky_of_frame, cudaStream_t st);
-// one radix pass over the keys of n_vals floats: histogram (256 bins, device,
-// zeroed here) of digit `shift` among keys whose bits under pmask equal prefix
-cudaError_t launch_key_histogram(const float *v, long long n_vals, uint32_t prefix, uint32_t pmask, int shift,
-                                 unsigned int *hist, cudaStream_t st);
-// FP64 sums: sums[0] += v, or with mean != null sums[1] += (v - *mean)^2
-cudaError_t launch_frame_sums(const float *v, long long n_vals, const double *mean, double *sums, cudaStream_t st);
-cudaError_t launch_bad_map(const float *ref, long long n_vals, const float *med, const double *thresh,
-                           uint8_t *map, cudaStream_t st);
-// bad pixel correction: mark (flagged or non-finite -> NaN), then passes
-cudaError_t launch_bad_mark(float *cube, long long T, int n, const uint8_t *map, unsigned long long *nan_count,
+// bad pixel map of the n_vals values of ref, in a device workspace of
+// bad_map_bytes(): FP64 sums, the exact median by three 11-bit digits of the
+// total-order keys, then the map; all on the stream, no host step between
+// (result: the first double of the workspace is the sum of the values)
+size_t bad_map_bytes();
+cudaError_t launch_bad_map(const float *ref, long long n_vals, double C, uint8_t *map, void *ws, cudaStream_t st);
+// bad pixel correction: the flagged and non-finite pixels become NaN and are
+// listed per frame (ws: n x n words a frame), then each frame with at most
+// n x n / 2 of them (n <= 65535) is filled from its list.  counts (device, fix_count_words(T)
+// u32): [0] frames with more (left to the dense passes), [1] pixels of other
+// frames that no pass can fill, [2..2+T) listed pixels
+size_t fix_count_words(long long T);
+cudaError_t launch_bad_fill(float *cube, long long T, int n, const uint8_t *map, uint32_t *ws, uint32_t *counts,
                             cudaStream_t st);
+// one dense pass: every NaN pixel of src with a finite 8-neighbour filled
+// into dst, the others copied; counts[0] += NaN left, counts[1] += filled
 cudaError_t launch_bad_pass(const float *src, float *dst, long long T, int n, unsigned long long *counts,
                             cudaStream_t st);
 

@@ -27,8 +27,11 @@
 // (collapse2_kernel); radix selects (8-bit digits) are its exact fallback and
 // the masked (master sky) and long-cube form (collapse_kernel).
 #include <cuda_runtime.h>
-#include <type_traits>
+#include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "graphic_internal.h"
 #include "select_common.cuh"
@@ -63,6 +66,24 @@ constexpr int COL_KS = 5;
 // 4-byte copies per frame)
 constexpr int C2_KS = 4;
 
+// Whether frame t's star mask covers pixel (col, row): (col - mask_x)^2 +
+// (row - mask_y)^2 < mask_r2 in FP64.  The same sum in FP32 decides unless it
+// lies within its own error of the bound (f.z = 4 E with E = 2^-23 (|mask_x|,
+// |mask_y| max + n) bounds the error of either difference, the rest is the
+// rounding of the squares, their sum and mask_r2); a mask too far off or not
+// finite has f.z = inf and always takes the FP64 sum.  GB300's FP64 pipe is
+// 1/64 of its FP32 one: the FP64 test of every value was most of the master
+// sky's time (290 us for 50 frames of 512 x 512, 262144 x 50 x 4 FP64
+// operations at about 2 per SM and cycle being 90 us of it).
+__device__ __forceinline__ bool mask_covers(const CollapseArgs &a, long long t, const float4 f, int col, int row) {
+  const float dx = (float)col - f.x, dy = (float)row - f.y;
+  const float d2 = fmaf(dx, dx, dy * dy), r2 = (float)a.mask_r2;
+  const float tol = f.z * (fabsf(dx) + fabsf(dy) + 1.0f) + 4.8e-7f * (d2 + r2);
+  if (fabsf(d2 - r2) > tol) return d2 < r2;
+  const double ex = (double)col - a.mask_x[t], ey = (double)row - a.mask_y[t];
+  return ex * ex + ey * ey < a.mask_r2;
+}
+
 // MASKED (master sky, Sect. 3.2): values that are not finite or fall in the
 // frame's star mask are left out -- they get the largest key, so they rank
 // after every value kept -- and the median is taken over the m values kept
@@ -94,8 +115,7 @@ __global__ void __launch_bounds__(32 * COL_PPC) collapse_kernel(const CollapseAr
     if constexpr (MASKED) {
       bool keep = isfinite(v);
       if (a.mask_x) {
-        const double ddx = (double)(p % a.n) - a.mask_x[t], ddy = (double)(p / a.n) - a.mask_y[t];
-        keep &= !(ddx * ddx + ddy * ddy < a.mask_r2);
+        keep &= !mask_covers(a, t, __ldg(&a.maskf[t]), (int)(p % a.n), (int)(p / a.n));
       }
       return keep ? f2key(v) : 0xffffffffu;
     } else {
@@ -226,6 +246,43 @@ __global__ void __launch_bounds__(32 * COL_PPC) collapse_kernel(const CollapseAr
     med = (lo + key2f(hi)) * 0.5f;
   }
   if (lane == 0) a.out[p] = med;
+}
+
+// Master sky of at most W frames (W <= 64): one thread per pixel, the values
+// in registers, the two middle ones by the pruned odd-even merge network
+// (middle_pair).  A value left out, like a slot beyond the last frame, is
+// replaced by +inf and -inf in turn, +inf first: the kept values stay in the
+// middle of the W slots (kept values are finite).  Reads every value once,
+// with all of a pixel's loads independent.  Bound by the instruction stream
+// (mask and finiteness tests and 612 of the 806 min / max of 403 comparators
+// per 50 values): 50 frames of 512 x 512 with masks in 30 us = 1.7 TB/s, where
+// the radix select with an FP64 mask test per value took 290 us.
+template <int W>
+__global__ void __launch_bounds__(128) sky_net_kernel(const CollapseArgs a) {
+  const int NN = a.n * a.n, T = (int)a.T;
+  const int p = blockIdx.x * 128 + threadIdx.x;
+  const int row = p / a.n, col = p - row * a.n;
+  float v[W];
+#pragma unroll
+  for (int i = 0; i < W; i++) v[i] = i < T ? __ldcs(a.in + (long long)i * NN + p) : INFINITY;
+  float pad = INFINITY;
+  int m = 0;
+#pragma unroll
+  for (int i = 0; i < W; i++) {
+    bool keep = i < T && isfinite(v[i]);
+    if (i < T && a.mask_x) {
+      // a warp's pixels share their row: most masks stay clear of it
+      const float4 f = __ldg(&a.maskf[i]);
+      if (fabsf((float)row - f.y) <= f.w) keep &= !mask_covers(a, i, f, col, row);
+    }
+    m += keep ? 1 : 0;
+    v[i] = keep ? v[i] : pad;
+    pad = keep ? pad : -pad;
+  }
+  middle_pair<W>(v);
+  const float lo = v[W / 2 - 1], hi = v[W / 2];
+  const float med = (m & 1) ? lo : (lo + hi) * 0.5f;
+  a.out[p] = m > 0 ? med : __uint_as_float(0x7fc00000u);   // no value left: NaN
 }
 
 // Median collapse of unmasked cubes that fit shared memory.  Per pixel
@@ -729,8 +786,25 @@ cudaError_t launch_collapse(const CollapseArgs &a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+float4 sky_mask_filter(double mask_x, double mask_y, double mask_r, int n) {
+  const double E = (std::max(fabs(mask_x), fabs(mask_y)) + n) * 0x1p-23;
+  if (!(E < 0.5)) return make_float4(0.f, 0.f, INFINITY, INFINITY);
+  return make_float4((float)mask_x, (float)mask_y, (float)(4.0 * E), (float)(mask_r * 1.000001 + 4.0 * E));
+}
+
 cudaError_t launch_sky_median(const CollapseArgs &a, cudaStream_t st) {
   const long long NN = (long long)a.n * a.n;
+  // up to 64 frames: the network that holds them, one thread per pixel (n a
+  // power of two from 64 on: whole blocks); longer stacks one warp per pixel
+  if (a.T <= 64) {
+    const unsigned blocks = (unsigned)(NN / 128);
+    if (a.T <= 8) sky_net_kernel<8><<<blocks, 128, 0, st>>>(a);
+    else if (a.T <= 16) sky_net_kernel<16><<<blocks, 128, 0, st>>>(a);
+    else if (a.T <= 32) sky_net_kernel<32><<<blocks, 128, 0, st>>>(a);
+    else if (a.T <= 50) sky_net_kernel<50><<<blocks, 128, 0, st>>>(a);
+    else sky_net_kernel<64><<<blocks, 128, 0, st>>>(a);
+    return cudaGetLastError();
+  }
   const unsigned grid = (unsigned)(NN / COL_PPC);
   if (a.T <= 8192) {
     const size_t smem = (size_t)(COL_PPC * 256 + COL_KS * a.T) * sizeof(uint32_t);
