@@ -54,6 +54,7 @@ struct graphic_ctx {
   size_t lparam_bytes = 0;
   char *d_gparam = nullptr;         // grouped executor: parameter tables, one region per branch
   size_t gparam_bytes = 0;
+  long long alloc_gen = 0;          // buffers (re)allocated so far
   bool prof = false;
   double prof_ms[GRAPHIC_K_COUNT] = {};
   int64_t prof_n[GRAPHIC_K_COUNT] = {};
@@ -140,8 +141,12 @@ int check_cube(const void *in, const void *out, int64_t T, int32_t n, bool devic
   return GRAPHIC_OK;
 }
 
-int ensure(void **ptr, size_t *have, size_t need, bool pinned) {
+// Grow a buffer of the context.  A recorded graph names the buffers it was
+// recorded with, and a new one may take the address of the one it replaces,
+// so every allocation counts in alloc_gen, which the graphs' keys hold.
+int ensure(graphic_ctx *c, void **ptr, size_t *have, size_t need, bool pinned) {
   if (*have >= need && *ptr) return GRAPHIC_OK;
+  c->alloc_gen++;
   if (*ptr) {
     if (pinned) cudaFreeHost(*ptr); else cudaFree(*ptr);
     *ptr = nullptr;
@@ -203,9 +208,9 @@ struct PlanBuilder {
 
 int upload_plan(graphic_ctx *c, const PlanBuilder &pb) {
   const size_t bytes = std::max<size_t>(pb.buf.size(), 16);
-  int rc = ensure((void **)&c->h_plan, &c->h_plan_bytes, bytes, true);
+  int rc = ensure(c, (void **)&c->h_plan, &c->h_plan_bytes, bytes, true);
   if (rc) return rc;
-  rc = ensure((void **)&c->d_plan, &c->d_plan_bytes, bytes, false);
+  rc = ensure(c, (void **)&c->d_plan, &c->d_plan_bytes, bytes, false);
   if (rc) return rc;
   memcpy(c->h_plan, pb.buf.data(), pb.buf.size());
   CK(cudaMemcpyAsync(c->d_plan, c->h_plan, pb.buf.size(), cudaMemcpyHostToDevice, c->stream));
@@ -276,7 +281,7 @@ int enqueue_shift(graphic_ctx *c, const float *in, float *out, int64_t T, int32_
   const long long ch = chunk_frames(c, T, (size_t)NN * sizeof(float));
   // per-frame shift parameters of both passes, once for all frames
   const size_t pb = line_params_bytes(SHIFT_X, n, T);
-  int rc = ensure((void **)&c->d_lparam, &c->lparam_bytes, 2 * pb, false);
+  int rc = ensure(c, (void **)&c->d_lparam, &c->lparam_bytes, 2 * pb, false);
   if (rc) return rc;
   {
     LineArgs a{};
@@ -350,11 +355,11 @@ int enqueue_rotate(graphic_ctx *c, const float *in, float *out, int64_t T, int32
   if (!in_fs) in_fs = NN;
   if (!out_fs) out_fs = NN;
   const long long ch = chunk_frames(c, T, (size_t)NM * sizeof(float));
-  int rc = ensure((void **)&c->d_scratch, &c->scratch_bytes, (size_t)ch * NM * sizeof(float), false);
+  int rc = ensure(c, (void **)&c->d_scratch, &c->scratch_bytes, (size_t)ch * NM * sizeof(float), false);
   if (rc) return rc;
   // per-line shear parameters of a chunk: passes 1 and 3 share theirs
   const size_t pb13 = line_params_bytes(ROT_P1, n, ch), pb2 = line_params_bytes(ROT_P2, n, ch);
-  if ((rc = ensure((void **)&c->d_lparam, &c->lparam_bytes, pb13 + pb2, false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_lparam, &c->lparam_bytes, pb13 + pb2, false))) return rc;
   for (long long f0 = 0; f0 < T; f0 += ch) {
     const long long nf = std::min<long long>(ch, T - f0);
     LineArgs a{};
@@ -655,7 +660,7 @@ int enqueue_adi(graphic_ctx *c, const float *in, float *out, int64_t T, int32_t 
   for (int64_t t = 0; t < T && perm_id; t++) perm_id = ap.perm[t] == (int)t;
   const size_t need = band_scratch_bytes(ap, T);
   if (need) {
-    int rc = ensure((void **)&c->d_bscratch, &c->bscratch_bytes, need, false);
+    int rc = ensure(c, (void **)&c->d_bscratch, &c->bscratch_bytes, need, false);
     if (rc) return rc;
   }
   return enqueue_adi_raw(c, in, out, T, n, at<int>(c, o.perm), at<int>(c, o.lr), at<double>(c, o.e2),
@@ -853,7 +858,7 @@ int batch_persistent(graphic_ctx *c, const graphic_batch_item *items, int32_t n_
     wave_max = std::max(wave_max, used);
   }
   waves++;
-  int rc = ensure((void **)&c->d_scratch, &c->scratch_bytes, 2 * wave_max, false);
+  int rc = ensure(c, (void **)&c->d_scratch, &c->scratch_bytes, 2 * wave_max, false);
   if (rc) return rc;
   for (int f = 0; f < nframes; f++)
     fr[f].scratch = c->d_scratch + ((fr[f].wave & 1) ? wave_max / sizeof(float) : 0) + wave_off[f] / sizeof(float);
@@ -884,11 +889,11 @@ int batch_persistent(graphic_ctx *c, const graphic_batch_item *items, int32_t n_
   const size_t o_w = pb.add(wave_r3.data(), wave_r3.size() * sizeof(int));
   const size_t o_si = pb.add(seg_of_item.data(), seg_of_item.size() * sizeof(int));
   const size_t cbytes = sizeof(int) * (1 + 5 * (size_t)nframes + waves);
-  if ((rc = ensure((void **)&c->d_counters, &c->counters_bytes, cbytes, false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_counters, &c->counters_bytes, cbytes, false))) return rc;
   // the pinned / device plan buffers must not move under a recorded graph
   const size_t pbytes = std::max<size_t>(pb.buf.size(), 16);
-  if ((rc = ensure((void **)&c->h_plan, &c->h_plan_bytes, pbytes, true))) return rc;
-  if ((rc = ensure((void **)&c->d_plan, &c->d_plan_bytes, pbytes, false))) return rc;
+  if ((rc = ensure(c, (void **)&c->h_plan, &c->h_plan_bytes, pbytes, true))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_plan, &c->d_plan_bytes, pbytes, false))) return rc;
   memcpy(c->h_plan, pb.buf.data(), pb.buf.size());
   BatchArgs b{};
   b.frames = reinterpret_cast<const BatchFrame *>(c->d_plan + o_fr);
@@ -907,7 +912,7 @@ int batch_persistent(graphic_ctx *c, const graphic_batch_item *items, int32_t n_
                                       (long long)pb.buf.size(), (long long)o_sg, (long long)o_w, (long long)o_si,
                                       (long long)(uintptr_t)c->d_counters, (long long)cbytes, b.nseg, b.total,
                                       nframes, (long long)(uintptr_t)c->d_status, c->batch_ctas_per_sm,
-                                      (long long)(uintptr_t)c->stream};
+                                      (long long)(uintptr_t)c->stream, c->alloc_gen};
   if (c->graph_exec && key != c->graph_key) {
     cudaGraphExecDestroy(c->graph_exec);
     cudaGraphDestroy(c->graph);
@@ -1020,7 +1025,7 @@ int batch_grouped(graphic_ctx *c, const graphic_batch_item *items, int32_t n_ite
   }
   const int R = std::max(1, std::min<int>(c->group_streams, (int)waves.size()));
   int rc;
-  if (slot_bytes && (rc = ensure((void **)&c->d_gscratch, &c->gscratch_bytes, slot_bytes * R, false))) return rc;
+  if (slot_bytes && (rc = ensure(c, (void **)&c->d_gscratch, &c->gscratch_bytes, slot_bytes * R, false))) return rc;
   // per-line shift parameter tables of a wave (one region per branch):
   // shift x and y per frame, then shears of rotation passes 1/3 and 2
   auto wave_tab_bytes = [](const GroupWave &w) -> size_t {
@@ -1033,7 +1038,7 @@ int batch_grouped(graphic_ctx *c, const graphic_batch_item *items, int32_t n_ite
   size_t tab_bytes = 16;
   for (const GroupWave &w : waves) tab_bytes = std::max(tab_bytes, wave_tab_bytes(w));
   tab_bytes = (tab_bytes + 255) & ~(size_t)255;
-  if ((rc = ensure((void **)&c->d_gparam, &c->gparam_bytes, tab_bytes * R, false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_gparam, &c->gparam_bytes, tab_bytes * R, false))) return rc;
   // plan: per frame tables in the sorted order
   std::vector<const float *> tin(nframes), trin(nframes);
   std::vector<float *> tout(nframes);
@@ -1059,14 +1064,14 @@ int batch_grouped(graphic_ctx *c, const graphic_batch_item *items, int32_t n_ite
   const size_t o_s = pb.add(ps.data(), nframes * sizeof(double));
   const size_t o_q = pb.add(pq.data(), nframes * sizeof(int));
   const size_t pbytes = std::max<size_t>(pb.buf.size(), 16);
-  if ((rc = ensure((void **)&c->h_plan, &c->h_plan_bytes, pbytes, true))) return rc;
-  if ((rc = ensure((void **)&c->d_plan, &c->d_plan_bytes, pbytes, false))) return rc;
+  if ((rc = ensure(c, (void **)&c->h_plan, &c->h_plan_bytes, pbytes, true))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_plan, &c->d_plan_bytes, pbytes, false))) return rc;
   memcpy(c->h_plan, pb.buf.data(), pb.buf.size());
   std::vector<long long> key = {(long long)(uintptr_t)c->h_plan, (long long)(uintptr_t)c->d_plan,
                                 (long long)pb.buf.size(), (long long)(uintptr_t)c->d_gscratch, (long long)slot_bytes,
                                 (long long)(uintptr_t)c->d_status, R, c->variant_1024, c->precision,
                                 (long long)(uintptr_t)c->stream, (long long)(uintptr_t)c->d_gparam,
-                                (long long)tab_bytes};
+                                (long long)tab_bytes, c->alloc_gen};
   for (const GroupWave &w : waves) {
     key.push_back(w.n);
     key.push_back(w.mask);
@@ -1515,8 +1520,8 @@ int graphic_reduce_host(graphic_ctx *c, const float *host_in, int64_t T, int32_t
   if (T < 1) return fail(GRAPHIC_ERR_INVALID_ARG, "n_frames < 1");
   DeviceGuard g(c->device);
   const size_t NN = (size_t)n * n;
-  if ((rc = ensure((void **)&c->d_cube, &c->cube_bytes, (size_t)T * NN * sizeof(float), false))) return rc;
-  if ((rc = ensure((void **)&c->d_img, &c->img_bytes, NN * sizeof(float), false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_cube, &c->cube_bytes, (size_t)T * NN * sizeof(float), false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_img, &c->img_bytes, NN * sizeof(float), false))) return rc;
   if ((rc = reduce_device(c, c->d_cube, c->d_cube, T, n, dx, dy, parang, fwhm, n_fwhm, edges, n_edges, c->d_img,
                           host_in))) {
     cudaStreamSynchronize(c->stream);
@@ -1815,7 +1820,7 @@ int graphic_bad_pixel_map(graphic_ctx *c, const float *ref, int32_t n, double C,
   if (!std::isfinite(C) || C < 0) return fail(GRAPHIC_ERR_INVALID_ARG, "C must be finite, >= 0");
   DeviceGuard g(c->device);
   int rc;
-  if ((rc = ensure((void **)&c->d_prep, &c->prep_bytes, std::max<size_t>(4096, bad_map_bytes()), false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_prep, &c->prep_bytes, std::max<size_t>(4096, bad_map_bytes()), false))) return rc;
   cudaError_t e = launch_bad_map(ref, (long long)n * n, C, map, c->d_prep, c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "bad pixel map kernels");
   volatile double *sum = reinterpret_cast<volatile double *>(c->h_status + 2);
@@ -1832,8 +1837,8 @@ int graphic_bad_pixel_fix(graphic_ctx *c, float *cube, int64_t T, int32_t n, con
   DeviceGuard g(c->device);
   const size_t bytes = (size_t)T * n * n * sizeof(float);
   int rc;
-  if ((rc = ensure((void **)&c->d_prep, &c->prep_bytes, 4096 + fix_count_words(T) * sizeof(uint32_t), false))) return rc;
-  if ((rc = ensure((void **)&c->d_scratch, &c->scratch_bytes, bytes, false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_prep, &c->prep_bytes, 4096 + fix_count_words(T) * sizeof(uint32_t), false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_scratch, &c->scratch_bytes, bytes, false))) return rc;
   uint32_t *d_counts = reinterpret_cast<uint32_t *>(c->d_prep + 4096);
   cudaError_t e = launch_bad_fill(cube, T, n, map, reinterpret_cast<uint32_t *>(c->d_scratch), d_counts, c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "bad pixel correction kernels");
@@ -1877,7 +1882,7 @@ int graphic_register(graphic_ctx *c, const float *in, int64_t T, int32_t n, doub
   if (T == 0) return GRAPHIC_OK;
   DeviceGuard g(c->device);
   int rc;
-  if ((rc = ensure((void **)&c->d_scratch, &c->scratch_bytes, register_keys_bytes(T), false))) return rc;
+  if ((rc = ensure(c, (void **)&c->d_scratch, &c->scratch_bytes, register_keys_bytes(T), false))) return rc;
   if ((rc = begin_call(c))) return rc;
   RegArgs a;
   a.in = in;
@@ -1997,7 +2002,7 @@ int graphic_aperture(graphic_ctx *c, const float *img, int32_t n, int32_t n_ap, 
   PlanBuilder pb;
   const size_t o_xy = pb.add(xy.data(), xy.size() * sizeof(double));
   int rc;
-  if ((rc = ensure((void **)&c->d_prep, &c->prep_bytes, std::max<size_t>(4096, (size_t)n_ap * sizeof(double)),
+  if ((rc = ensure(c, (void **)&c->d_prep, &c->prep_bytes, std::max<size_t>(4096, (size_t)n_ap * sizeof(double)),
                    false)))
     return rc;
   if ((rc = begin_call(c))) return rc;
