@@ -180,8 +180,8 @@ int graphic_reduce_cube(graphic_ctx *ctx, const graphic_cube *in, const graphic_
  * times must be monotone along the order of the parallactic angles (as for
  * a transit observed in time order), else GRAPHIC_ERR_UNSUPPORTED; t_max
  * must be > 0 (GRAPHIC_ERR_INVALID_ARG).  With a time condition every pixel
- * takes the general median path (sort + membership sweep), not the faster
- * band path.
+ * takes the general median path (every frame ranked), not the faster band
+ * path.
  */
 int graphic_adi_subtract_ex(graphic_ctx *ctx, const float *in, float *out, int64_t n_frames, int32_t n,
                             const double *parang, const double *times, double t_max, double fwhm, double n_fwhm,

@@ -574,7 +574,7 @@ namespace {
 
 // Plan tables of the median PSF step in the uploaded plan (byte offsets).
 struct AdiOffsets {
-  size_t perm, lr, e2, band, ab, evq, groups;
+  size_t perm, lr, e2, band, ab, evq, groups, units, zero;
 };
 
 AdiOffsets add_adi_plan(PlanBuilder &pb, const AdiPlanHost &ap, int64_t T) {
@@ -586,53 +586,10 @@ AdiOffsets add_adi_plan(PlanBuilder &pb, const AdiPlanHost &ap, int64_t T) {
   o.ab = pb.add(ap.ab.data(), ap.ab.size() * sizeof(int));
   o.evq = pb.add(ap.evq.data(), ap.evq.size() * sizeof(uint32_t));
   o.groups = pb.add(ap.groups.data(), ap.groups.size() * sizeof(int));
+  o.units = pb.add(ap.units.data(), ap.units.size() * sizeof(int));
+  o.zero = pb.add(ap.zero.data(), ap.zero.size() * sizeof(int));
   return o;
 }
-
-int enqueue_adi_raw(graphic_ctx *c, const float *in, float *out, int64_t T, int32_t n, const int *p_perm,
-                    const int *p_lr, const double *p_edge2, const int *p_band, int wmax, int n_ann,
-                    const int *p_ab, const uint32_t *p_evq, const int *p_groups, const std::vector<int> &class_off,
-                    int gen_off, int gen_n, char *band_scratch, size_t band_scratch_cap, long long in_fs,
-                    long long out_fs, bool perm_id) {
-  AdiArgs a{};
-  a.perm_id = perm_id ? 1 : 0;
-  a.in_fs = in_fs ? in_fs : (long long)n * n;
-  a.out_fs = out_fs ? out_fs : (long long)n * n;
-  a.band_scratch_cap = band_scratch_cap;
-  a.evq = p_evq;
-  a.groups = p_groups;
-  for (int k = 0; k < 8; k++) a.class_off[k] = k < (int)class_off.size() ? class_off[k] : 0;
-  a.gen_list = gen_off >= 0 ? 1 : 0;
-  a.gen_off = gen_off;
-  a.gen_n = gen_n;
-  a.band_scratch = band_scratch;
-  a.in = in;
-  a.out = out;
-  a.perm = p_perm;
-  a.lr = p_lr;
-  a.ab = p_ab;
-  a.edge2 = p_edge2;
-  a.band = p_band;
-  a.wmax = wmax;
-  a.status = c->d_status;
-  a.T = (int)T;
-  a.n = n;
-  a.n_ann = n_ann;
-  // profiling: one bracket per group of launches (general path, band
-  // preparation with the zero groups, band sweep)
-  a.mark_user = c;
-  a.mark = [](void *u, int kind, int begin) {
-    graphic_ctx *cc = static_cast<graphic_ctx *>(u);
-    const int id = kind == 0 ? GRAPHIC_K_ADI_MEDIAN : kind == 1 ? GRAPHIC_K_ADI_BAND_PREP : GRAPHIC_K_ADI_BAND_SWEEP;
-    if (begin) prof_begin(cc, id);
-    else prof_end(cc);
-  };
-  int launched = 0;
-  cudaError_t e = launch_adi_median(a, c->stream, &launched);
-  if (e != cudaSuccess) return cuda_fail(e, "median PSF kernel");
-  return GRAPHIC_OK;
-}
-
 
 int enqueue_collapse(graphic_ctx *c, const float *in, int64_t T, int32_t n, float *out, long long in_fs = 0) {
   CollapseArgs a{};
@@ -658,16 +615,48 @@ int enqueue_adi(graphic_ctx *c, const float *in, float *out, int64_t T, int32_t 
                 const AdiOffsets &o, long long in_fs = 0, long long out_fs = 0) {
   bool perm_id = true;
   for (int64_t t = 0; t < T && perm_id; t++) perm_id = ap.perm[t] == (int)t;
-  const size_t need = band_scratch_bytes(ap, T);
+  const size_t need = psf_scratch_bytes(ap, T);
   if (need) {
     int rc = ensure(c, (void **)&c->d_bscratch, &c->bscratch_bytes, need, false);
     if (rc) return rc;
   }
-  return enqueue_adi_raw(c, in, out, T, n, at<int>(c, o.perm), at<int>(c, o.lr), at<double>(c, o.e2),
-                         at<int>(c, o.band), ap.wmax, (int)ap.edge2.size() - 1,
-                         ap.ab.empty() ? nullptr : at<int>(c, o.ab), at<uint32_t>(c, o.evq), at<int>(c, o.groups),
-                         ap.class_off, ap.gen_off, ap.gen_n, c->d_bscratch, c->bscratch_bytes, in_fs, out_fs,
-                         perm_id);
+  AdiArgs a{};
+  a.perm_id = perm_id ? 1 : 0;
+  a.in_fs = in_fs ? in_fs : (long long)n * n;
+  a.out_fs = out_fs ? out_fs : (long long)n * n;
+  a.band_scratch = c->d_bscratch;
+  a.band_scratch_cap = c->bscratch_bytes;
+  a.wmax = ap.wmax;
+  a.evq = at<uint32_t>(c, o.evq);
+  a.groups = at<int>(c, o.groups);
+  for (int k = 0; k < 8; k++) a.class_off[k] = k < (int)ap.class_off.size() ? ap.class_off[k] : 0;
+  a.units = at<int>(c, o.units);
+  a.n_units = (int)ap.units.size() / 4;
+  a.zero = at<int>(c, o.zero);
+  a.n_zero = (int)ap.zero.size();
+  a.in = in;
+  a.out = out;
+  a.perm = at<int>(c, o.perm);
+  a.lr = at<int>(c, o.lr);
+  a.ab = ap.ab.empty() ? nullptr : at<int>(c, o.ab);
+  a.edge2 = at<double>(c, o.e2);
+  a.band = at<int>(c, o.band);
+  a.status = c->d_status;
+  a.T = (int)T;
+  a.n = n;
+  a.n_ann = (int)ap.edge2.size() - 1;
+  // profiling: one bracket per group of launches (general path, band
+  // preparation with the zero groups, band sweep)
+  a.mark_user = c;
+  a.mark = [](void *u, int kind, int begin) {
+    graphic_ctx *cc = static_cast<graphic_ctx *>(u);
+    const int id = kind == 0 ? GRAPHIC_K_ADI_MEDIAN : kind == 1 ? GRAPHIC_K_ADI_BAND_PREP : GRAPHIC_K_ADI_BAND_SWEEP;
+    if (begin) prof_begin(cc, id);
+    else prof_end(cc);
+  };
+  cudaError_t e = launch_adi_median(a, c->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "median PSF kernel");
+  return GRAPHIC_OK;
 }
 
 // Full reduction of the device cube `in` (work may equal in).  With host_in,
@@ -686,7 +675,7 @@ int reduce_device(graphic_ctx *c, const float *in, float *work, int64_t T, int32
   if (rc) return rc;
   AdiPlanHost ap;
   if ((rc = plan_adi(parang, T, fwhm, n_fwhm, edges, n_edges, ap, times, t_max))) return rc;
-  if ((rc = plan_band_path(ap, T, n))) return rc;
+  if ((rc = plan_band_path(ap, T, n)) || (rc = plan_general_path(ap, T, n))) return rc;
   PlanBuilder pb;
   const size_t o_dx = pb.add(dx, T * sizeof(double));
   const size_t o_dy = pb.add(dy, T * sizeof(double));
@@ -1462,7 +1451,7 @@ int graphic_adi_subtract_ex(graphic_ctx *c, const float *in, float *out, int64_t
   if ((rc = validate_adi(parang, T, fwhm, n_fwhm, edges, n_edges))) return rc;
   AdiPlanHost ap;
   if ((rc = plan_adi(parang, T, fwhm, n_fwhm, edges, n_edges, ap, times, t_max))) return rc;
-  if ((rc = plan_band_path(ap, T, n))) return rc;
+  if ((rc = plan_band_path(ap, T, n)) || (rc = plan_general_path(ap, T, n))) return rc;
   DeviceGuard g(c->device);
   PlanBuilder pb;
   const AdiOffsets oa = add_adi_plan(pb, ap, T);
@@ -1608,7 +1597,7 @@ int graphic_adi_subtract_cube(graphic_ctx *c, const graphic_cube *in, const grap
   if ((rc = validate_adi(parang, T, fwhm, n_fwhm, edges, n_edges))) return rc;
   AdiPlanHost ap;
   if ((rc = plan_adi(parang, T, fwhm, n_fwhm, edges, n_edges, ap))) return rc;
-  if ((rc = plan_band_path(ap, T, n))) return rc;
+  if ((rc = plan_band_path(ap, T, n)) || (rc = plan_general_path(ap, T, n))) return rc;
   DeviceGuard g(c->device);
   PlanBuilder pb;
   const AdiOffsets oa = add_adi_plan(pb, ap, T);

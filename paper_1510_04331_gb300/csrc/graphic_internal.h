@@ -65,26 +65,32 @@ struct AdiPlanHost {
   // band path (plan_band_path): event queries [A][T] (a_s | b_s << 16: frame s
   // is outside the reference set of the queries a_s <= i < b_s), the 4-pixel
   // groups of the band path class after class (0: no pixel in an annulus;
-  // then bit map widths 1, 2, 4, 8, 16, 32 words), class offsets [8]; after
-  // the classes, from gen_off on, the gen_n 8-pixel blocks (index p / 8)
-  // with a pixel of an annulus that has no band: the general path's grid
-  // (gen_off < 0: every block)
+  // then bit map widths 1, 2, 4, 8, 16, 32 words), class offsets [8]
   std::vector<uint32_t> evq;
   std::vector<int> groups;
   std::vector<int> class_off;
-  int gen_off = -1, gen_n = 0;
+  // general path (plan_general_path): units of 32 pixels of one annulus, 4
+  // ints a unit (segments of 8 adjacent pixels, -1: none; the first also
+  // holds the annulus), and the segments with a pixel it sets to zero
+  std::vector<int> units, zero;
 };
 // Returns GRAPHIC_OK, or an error code (last error set) for times that are
 // not monotone in the angle order or a t_max that is not > 0.
 int plan_adi(const double *parang, int64_t T, double fwhm, double n_fwhm, const double *edges, int32_t n_edges,
              AdiPlanHost &ap, const double *times = nullptr, double t_max = 0.0);
-// Band path tables of a plan for frames of side n (psf_band.cu); the groups
-// of a geometry are cached.  band_scratch_bytes: the device scratch the band
-// path of that plan needs.
+// Band path tables of a plan for frames of side n (psf_band.cu) and general
+// path units (psf_general.cu); the lists of a geometry are cached.
+// psf_scratch_bytes: the device scratch the two need, one after the other.
 int plan_band_path(AdiPlanHost &ap, int64_t T, int32_t n);
+int plan_general_path(AdiPlanHost &ap, int64_t T, int32_t n);
 size_t band_scratch_bytes(const AdiPlanHost &ap, int64_t T);
-// The band path works through its pixel groups in chunks whose tables fit
-// the scratch it is given; kBandScratchMax bounds what callers allocate.
+size_t general_scratch_bytes(const AdiPlanHost &ap, int64_t T);
+inline size_t psf_scratch_bytes(const AdiPlanHost &ap, int64_t T) {
+  const size_t b = band_scratch_bytes(ap, T), g = general_scratch_bytes(ap, T);
+  return b > g ? b : g;
+}
+// Both work through their pixels in chunks whose tables fit the scratch they
+// are given; kBandScratchMax bounds what callers allocate.
 constexpr size_t kBandScratchMax = (size_t)256 << 20;
 
 // Asynchronous context calls for the serving loop (capi.cu): a batch call on
@@ -162,7 +168,7 @@ bool tc_supported(int n);
 cudaError_t launch_line_pass_tc(LineKind kind, const LineArgs &a, long long n_frames, cudaStream_t st,
                                 int precision);
 
-// median.cu
+// median PSF
 struct AdiArgs {
   const float *in;
   float *out;
@@ -185,11 +191,13 @@ struct AdiArgs {
   const uint32_t *evq;   // [A][T] device
   const int *groups;     // device, class after class
   int class_off[8];      // host copy of AdiPlanHost::class_off
-  int gen_list;          // 1: the general path runs on the gen_n blocks listed at groups + gen_off
-                         // (AdiPlanHost::gen_off, gen_n); 0: on every 8-pixel block
-  int gen_off, gen_n;
-  char *band_scratch;    // device scratch of band_scratch_cap bytes (at least one group's tables)
-  size_t band_scratch_cap;
+  // general path (psf_general.cu), from plan_general_path
+  const int *units;      // device
+  int n_units;
+  const int *zero;       // device
+  int n_zero;
+  char *band_scratch;    // device scratch of band_scratch_cap bytes (at least psf_scratch_bytes or
+  size_t band_scratch_cap;   // kBandScratchMax), used by one path after the other
   // optional hook around each group of launches (profiling): mark(user,
   // kind, 1) before and mark(user, kind, 0) after; kind 0 = general path,
   // 1 = band preparation (and the zero groups), 2 = band sweep
@@ -197,12 +205,13 @@ struct AdiArgs {
   void *mark_user;
 };
 // *launched (may be null) receives the number of kernels launched (the
-// general path when it has blocks, then the band path's launches).
+// general path's, then the band path's).
 cudaError_t launch_adi_median(const AdiArgs &a, cudaStream_t st, int *launched = nullptr);
 // psf_band.cu: the band path's launches (zero groups, then per class the
 // preparation and the sweep); *launched is incremented per kernel
 cudaError_t launch_adi_band(const AdiArgs &a, cudaStream_t st, int *launched);
 
+// median.cu
 struct CollapseArgs {
   const float *in;
   float *out;

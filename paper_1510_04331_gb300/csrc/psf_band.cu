@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(32 * PPC, 4) band_prep_kernel(const BandArgs B
     orv = __reduce_or_sync(FULL, orv);
     andv = __reduce_and_sync(FULL, andv);
     uint32_t Klo, Khi, clt_lo, clt_hi;
-    band_select2<KS>(kw, T, (uint32_t)blo, (uint32_t)bhi, orv ^ andv, andv, hist, cur, lane, Klo, clt_lo, Khi,
+    band_select2([&](int s) { return kw[s * KS]; }, T, (uint32_t)blo, (uint32_t)bhi, orv ^ andv, andv, hist, cur, lane, Klo, clt_lo, Khi,
                       clt_hi);
     const int need_lo = blo - (int)clt_lo;
     const int lim_hi = bhi + 1 - (int)clt_hi;
@@ -687,7 +687,6 @@ struct GroupKey {
 std::mutex g_group_mu;
 struct GroupLists {
   std::vector<int> groups, class_off;
-  int gen_off, gen_n;
 };
 std::map<GroupKey, GroupLists> g_group_cache;
 
@@ -698,8 +697,6 @@ int plan_band_path(AdiPlanHost &ap, int64_t T, int32_t n) {
   ap.evq.clear();
   ap.groups.clear();
   ap.class_off.assign(NCLASS + 1, 0);
-  ap.gen_off = -1;
-  ap.gen_n = 0;
   if (ap.wmax == 0 || A <= 0) return GRAPHIC_OK;
   // event queries of every banded annulus: frame s is outside S_i for
   // a_s <= i < b_s (two pointers over the monotone gates)
@@ -723,14 +720,11 @@ int plan_band_path(AdiPlanHost &ap, int64_t T, int32_t n) {
     if (it != g_group_cache.end()) {
       ap.groups = it->second.groups;
       ap.class_off = it->second.class_off;
-      ap.gen_off = it->second.gen_off;
-      ap.gen_n = it->second.gen_n;
       return GRAPHIC_OK;
     }
   }
   const int64_t NN = (int64_t)n * n;
   std::vector<std::vector<int>> lists(NCLASS);
-  std::vector<int> gen_blocks;   // 8-pixel blocks of the general path
   for (int64_t g = 0; g < NN / PPC; g++) {
     int cls = 0;
     bool general = false;
@@ -749,20 +743,16 @@ int plan_band_path(AdiPlanHost &ap, int64_t T, int32_t n) {
       if (W == 0) general = true;
       else cls = std::max(cls, class_of_width(W));
     }
-    if (!general) lists[cls].push_back((int)g);
-    else if (gen_blocks.empty() || gen_blocks.back() != (int)(g / 2)) gen_blocks.push_back((int)(g / 2));
+    if (!general) lists[cls].push_back((int)g);   // else psf_general.cu's
   }
   for (int k = 0; k < NCLASS; k++) {
     ap.class_off[k] = (int)ap.groups.size();
     ap.groups.insert(ap.groups.end(), lists[k].begin(), lists[k].end());
   }
   ap.class_off[NCLASS] = (int)ap.groups.size();
-  ap.gen_off = (int)ap.groups.size();
-  ap.gen_n = (int)gen_blocks.size();
-  ap.groups.insert(ap.groups.end(), gen_blocks.begin(), gen_blocks.end());
   std::lock_guard<std::mutex> lk(g_group_mu);
   if (g_group_cache.size() > 16) g_group_cache.clear();
-  g_group_cache[key] = {ap.groups, ap.class_off, ap.gen_off, ap.gen_n};
+  g_group_cache[key] = {ap.groups, ap.class_off};
   return GRAPHIC_OK;
 }
 

@@ -1,6 +1,6 @@
 // select_common.cuh -- device helpers shared by the selection kernels (the
-// median collapse and general median PSF path of median.cu, the band path of
-// psf_band.cu): IEEE total-order keys, asynchronous shared-memory copies, bit
+// median collapse and master sky of median.cu, the median PSF of psf_band.cu
+// and psf_general.cu, the binning of photometry.cu): IEEE total-order keys, asynchronous shared-memory copies, bit
 // selection.  Each translation unit gets its own copy (anonymous namespace).
 #pragma once
 
@@ -163,12 +163,12 @@ __device__ __forceinline__ void hist_find(const uint32_t *hist, uint32_t krem, i
 
 
 // Exact radix selects of the elements of full ranks r_lo <= r_hi among the T
-// keys keys[s * STRIDE] (s < T), sharing each histogram pass while both
-// prefixes agree: returns their keys and the numbers of smaller keys.
+// keys key_at(s) (s < T), sharing each histogram pass while both prefixes
+// agree: returns their keys and the numbers of smaller keys.
 // Histograms use fire-and-forget shared-memory reductions (no dependency
 // chain); digits equal in every key are skipped.
-template <int STRIDE>
-__device__ __forceinline__ void band_select2(const uint32_t *keys, int T, uint32_t r_lo, uint32_t r_hi,
+template <class KeyAt>
+__device__ __forceinline__ void band_select2(KeyAt key_at, int T, uint32_t r_lo, uint32_t r_hi,
                                              uint32_t varying, uint32_t andv, uint32_t *hlo, uint32_t *hhi,
                                              int lane, uint32_t &Klo, uint32_t &clt_lo, uint32_t &Khi,
                                              uint32_t &clt_hi) {
@@ -191,7 +191,7 @@ __device__ __forceinline__ void band_select2(const uint32_t *keys, int T, uint32
     __syncwarp();
 #pragma unroll 4
     for (int s = lane; s < T; s += 32) {
-      const uint32_t key = keys[s * STRIDE];
+      const uint32_t key = key_at(s);
       const uint32_t d = (key >> shift) & 255u;
       const uint32_t km = key & pmask;
       if (km == plo) atomicAdd(&hlo[d], 1u);

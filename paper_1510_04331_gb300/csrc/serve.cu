@@ -115,7 +115,7 @@ struct Req {
   // (plan_dev_bytes: the plan's device region, the staged tables)
   size_t cube_bytes = 0, out_bytes = 0, plan_bytes = 0, plan_dev_bytes = 0;
   size_t off_cube = Arena::kNone, off_out = Arena::kNone, off_plan = Arena::kNone;
-  size_t o_perm = 0, o_lr = 0, o_e2 = 0, o_band = 0, o_evq = 0, o_groups = 0;   // within the plan
+  size_t o_perm = 0, o_lr = 0, o_e2 = 0, o_band = 0, o_evq = 0, o_groups = 0, o_units = 0, o_zero = 0;   // within the plan
   size_t o_dx = 0, o_dy = 0;   // staged shifts
   size_t o_ptab = 0;           // device only (after the staged part): the shift passes' parameter tables
   // pinned staging: plan copy-in, result copy-out
@@ -274,6 +274,8 @@ int start_copy_in(graphic_server *s, Req *r) {
   memcpy(hp + r->o_band, r->ap.band.data(), r->ap.band.size() * sizeof(int));
   memcpy(hp + r->o_evq, r->ap.evq.data(), r->ap.evq.size() * sizeof(uint32_t));
   memcpy(hp + r->o_groups, r->ap.groups.data(), r->ap.groups.size() * sizeof(int));
+  memcpy(hp + r->o_units, r->ap.units.data(), r->ap.units.size() * sizeof(int));
+  memcpy(hp + r->o_zero, r->ap.zero.data(), r->ap.zero.size() * sizeof(int));
   memcpy(hp + r->o_dx, r->dx.data(), T * sizeof(double));
   memcpy(hp + r->o_dy, r->dy.data(), T * sizeof(double));
   char *plan = s->d_arena + r->off_plan;
@@ -442,13 +444,14 @@ void issue_iteration(graphic_server *s) {
     a.lr = reinterpret_cast<const int *>(plan + r->o_lr);
     a.edge2 = reinterpret_cast<const double *>(plan + r->o_e2);
     a.band = reinterpret_cast<const int *>(plan + r->o_band);
+    a.units = reinterpret_cast<const int *>(plan + r->o_units);
+    a.zero = reinterpret_cast<const int *>(plan + r->o_zero);
+    a.n_zero = (int)r->ap.zero.size();
+    a.n_units = (int)r->ap.units.size() / 4;
     a.wmax = r->ap.wmax;
     a.evq = reinterpret_cast<const uint32_t *>(plan + r->o_evq);
     a.groups = reinterpret_cast<const int *>(plan + r->o_groups);
     for (int k = 0; k < 8; k++) a.class_off[k] = k < (int)r->ap.class_off.size() ? r->ap.class_off[k] : 0;
-    a.gen_list = r->ap.gen_off >= 0 ? 1 : 0;
-    a.gen_off = r->ap.gen_off;
-    a.gen_n = r->ap.gen_n;
     a.band_scratch = s->d_band;   // shared: the median launches run one after the other on s_comp
     a.band_scratch_cap = graphic::kBandScratchMax;
     a.status = s->d_status + r->slot;
@@ -610,7 +613,7 @@ int graphic_server_submit(graphic_server *s, const graphic_request *rq, int64_t 
   r->theta.resize(T);
   for (int64_t t = 0; t < T; t++) r->theta[t] = -rq->parang[t];
   if ((rc = graphic::plan_adi(rq->parang, T, rq->fwhm, rq->n_fwhm, rq->edges, rq->n_edges, r->ap)) ||
-      (rc = graphic::plan_band_path(r->ap, T, rq->n))) {
+      (rc = graphic::plan_band_path(r->ap, T, rq->n)) || (rc = graphic::plan_general_path(r->ap, T, rq->n))) {
     delete r;
     return rc;
   }
@@ -631,6 +634,10 @@ int graphic_server_submit(graphic_server *s, const graphic_request *rq, int64_t 
   o = align16(o + r->ap.evq.size() * sizeof(uint32_t));
   r->o_groups = o;
   o = align16(o + r->ap.groups.size() * sizeof(int));
+  r->o_units = o;
+  o = align16(o + r->ap.units.size() * sizeof(int));
+  r->o_zero = o;
+  o = align16(o + r->ap.zero.size() * sizeof(int));
   r->o_dx = o;
   o = align16(o + T * sizeof(double));
   r->o_dy = o;
