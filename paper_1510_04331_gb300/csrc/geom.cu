@@ -13,9 +13,9 @@
 // pair packed as one complex line z = a + i b (two real lines), handled by
 // m/16 threads holding 16 complex values in registers.  Forward FFT =
 // Stockham autosort stages of radix 16, 16 and m/256 (or 16, 8 for m = 128):
-// the first stage reads global memory straight into registers (input half
-// zero: pruned at compile time), later stages exchange through shared
-// memory (ping-pong buffers, one pad slot every 16 entries against bank
+// the first stage reads global memory straight into registers, columns through
+// shared memory (input half zero: pruned at compile time), later stages
+// exchange through shared memory (ping-pong buffers, one pad slot every 16 entries against bank
 // conflicts).  The middle step separates the two real spectra where the two
 // lines have different shifts (shear passes), multiplies by the phasors and
 // stores conj(V)/m; the inverse is then the same forward stages
@@ -36,16 +36,28 @@
 namespace graphic {
 namespace {
 
-// Twiddle tables W_m^e = exp(-i 2 pi e / m), e in [0, m), for m = 128..2048,
-// stored back to back at offset m - 128 (FP64 cos/sin rounded to FP32).
-constexpr int kTwTotal = 4096 - 128;
+// Twiddle tables (FP64 cos/sin rounded to FP32), one per stage, laid out so
+// that a warp's loads of one r are contiguous: thread k of the stage takes
+// entry [r][k].
+//   stage 1, radix 16: W_256^(r k), k < 16 (the same for every m >= 256)
+//   stage 1, radix 8 (m = 128): W_128^(r k), k < 16
+//   stage 2, radix m / 256: W_m^(r k), k < 256, for m = 512, 1024, 2048
+//   the radix-32 x 32 warp FFT (m = 1024): W_1024^(r lane), lane < 32
+// Gathered from one table W_m^e at e = r k m / (16 radix), the loads took as
+// many wavefronts as the exchanges, which bound the kernels (the L1's data
+// pipe 81 % busy in rotation pass 3 of n = 1024): 60 frames, passes 1 / 2 / 3
+// 547 / 1177 / 445 -> 413 / 901 / 316 us; 777 of n = 128, 64 / 107 / 64 -> 61 /
+// 98 / 59.
+constexpr int kTwS1 = 0, kTwS1b = 256, kTwS2 = 384;   // stage 2: m at kTwS2 + m - 512
+constexpr int kTwTotal = kTwS2 + 512 + 1024 + 2048;
 __device__ float2 d_twiddle[kTwTotal];
-// The twiddles of the radix-32 x 32 warp FFT (m = 1024), W_1024^(r lane) at
-// [r][lane] (the same values as d_twiddle): lane-contiguous, so each of the
-// 31 twiddle loads of a lane group is one coalesced 256-byte access.
 __device__ float2 d_tw1024_rl[32 * 32];
 
-__host__ __device__ constexpr int tw_off(int m) { return m - 128; }
+// Table of the stage that multiplies by W_(NS R)^(r k), k < NS: entry [r][k].
+template <int R, int NS>
+__host__ __device__ constexpr int tw_stage() {
+  return NS == 256 ? kTwS2 + R * 256 - 512 : (R == 16 ? kTwS1 : kTwS1b);
+}
 
 // complex helpers, line parameters and frame loads: line_common.cuh
 
@@ -55,7 +67,64 @@ __host__ __device__ constexpr int tw_off(int m) { return m - 128; }
 #define G_S16 0.38268343236508977173f
 #define G_R2 0.70710678118654752440f
 
-template <int J>
+// Complex sums on Blackwell's packed FP32 instructions: real and imaginary
+// part in one register pair, one instruction for both (the same IEEE
+// operation on each half, so the same bits as two scalar ones at half the
+// issue slots; quarter turns and twiddle products stay scalar).  PK: used for
+// lines of 512 points and more; with 24 resident warps on the shorter lines
+// the issue slots are not what binds, and pairing the registers costs more
+// (777 frames of n = 128 rotated: pass 3 62 -> 69 us packed; n = 64 38 -> 49).
+// 800 frames of n = 512: shift rows 601 -> 516 us, rotation pass 1 919 -> 862,
+// pass 3 726 -> 649, the column passes (bound by shared-memory wavefronts)
+// unchanged; n = 1024 2 to 3 %.  Four lines per thread with the two pairs in
+// the halves (no scalar butterfly left, 2029 instructions per pair against
+// 3167 in pass 2) took 241 registers, left 8 warps an SM and lost: shift rows
+// 661, pass 3 817 us.
+__device__ __forceinline__ unsigned long long pack2(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ float2 padd(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+__device__ __forceinline__ float2 psub(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+template <bool PK>
+__device__ __forceinline__ float2 xadd(float2 a, float2 b) {
+  if constexpr (PK) return padd(a, b);
+  else return cadd(a, b);
+}
+template <bool PK>
+__device__ __forceinline__ float2 xsub(float2 a, float2 b) {
+  if constexpr (PK) return psub(a, b);
+  else return csub(a, b);
+}
+// a c + b, the real factor c on both parts
+__device__ __forceinline__ float2 pfma(float2 a, float c, float2 b) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(make_float2(c, c))), "l"(pack2(b)));
+  return unpack2(r);
+}
+
+// (a.x + i a.y)(c - i s)
+template <bool PK>
+__device__ __forceinline__ float2 mul_cs(float2 a, float c, float s) {
+  if constexpr (PK) return pfma(a, c, make_float2(a.y * s, -a.x * s));
+  else return make_float2(fmaf(a.x, c, a.y * s), fmaf(a.y, c, -a.x * s));
+}
+
+template <int J, bool PK>
 __device__ __forceinline__ float2 mul_w16(float2 a) {
   constexpr int j = J & 15;
   if constexpr (j == 0) return a;
@@ -68,21 +137,22 @@ __device__ __forceinline__ float2 mul_w16(float2 a) {
     constexpr float sn[16] = {0.f, G_S16, G_R2, G_C16, 1.f, G_C16, G_R2, G_S16,
                               0.f, -G_S16, -G_R2, -G_C16, -1.f, -G_C16, -G_R2, -G_S16};
     constexpr float c = cs[j], s = sn[j];
-    // (a.x + i a.y)(c - i s)
-    return make_float2(fmaf(a.x, c, a.y * s), fmaf(a.y, c, -a.x * s));
+    return mul_cs<PK>(a, c, s);
   }
 }
 
+template <bool PK>
 __device__ __forceinline__ void dft2(float2 &a, float2 &b) {
   float2 t = a;
-  a = cadd(t, b);
-  b = csub(t, b);
+  a = xadd<PK>(t, b);
+  b = xsub<PK>(t, b);
 }
 
+template <bool PK>
 __device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 &a3) {
-  float2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
-  a0 = cadd(t0, t2);
-  a2 = csub(t0, t2);
+  float2 t0 = xadd<PK>(a0, a2), t1 = xsub<PK>(a0, a2), t2 = xadd<PK>(a1, a3), t3 = xsub<PK>(a1, a3);
+  a0 = xadd<PK>(t0, t2);
+  a2 = xsub<PK>(t0, t2);
   a1 = make_float2(t1.x + t3.y, t1.y - t3.x);  // t1 - i t3
   a3 = make_float2(t1.x - t3.y, t1.y + t3.x);  // t1 + i t3
 }
@@ -90,59 +160,54 @@ __device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 
 // In-place forward DFT of size R on a[0..R), natural order out.
 // R = R1 * R2 with n = R2 n1 + n2, k = k1 + R1 k2: inner DFT_R1 over n1,
 // twiddle W_R^(n2 k1), outer DFT_R2 over n2, then the index transpose.
-template <int R>
-__device__ __forceinline__ void dft(float2 (&a)[R]);
-
-template <>
-__device__ __forceinline__ void dft<2>(float2 (&a)[2]) { dft2(a[0], a[1]); }
-
-template <>
-__device__ __forceinline__ void dft<4>(float2 (&a)[4]) { dft4(a[0], a[1], a[2], a[3]); }
-
-template <>
-__device__ __forceinline__ void dft<8>(float2 (&a)[8]) {
-  dft4(a[0], a[2], a[4], a[6]);
-  dft4(a[1], a[3], a[5], a[7]);
-  a[3] = mul_w16<2>(a[3]);   // n2 = 1, k1 = 1: W8^1
-  a[5] = mul_w16<4>(a[5]);   // k1 = 2
-  a[7] = mul_w16<6>(a[7]);   // k1 = 3
-  dft2(a[0], a[1]);
-  dft2(a[2], a[3]);
-  dft2(a[4], a[5]);
-  dft2(a[6], a[7]);
-  // slot 2 k1 + k2 holds X[k1 + 4 k2]
-  float2 t[8];
+template <int R, bool PK>
+__device__ __forceinline__ void dft(float2 (&a)[R]) {
+  if constexpr (R == 2) {
+    dft2<PK>(a[0], a[1]);
+  } else if constexpr (R == 4) {
+    dft4<PK>(a[0], a[1], a[2], a[3]);
+  } else if constexpr (R == 8) {
+    dft4<PK>(a[0], a[2], a[4], a[6]);
+    dft4<PK>(a[1], a[3], a[5], a[7]);
+    a[3] = mul_w16<2, PK>(a[3]);   // n2 = 1, k1 = 1: W8^1
+    a[5] = mul_w16<4, PK>(a[5]);   // k1 = 2
+    a[7] = mul_w16<6, PK>(a[7]);   // k1 = 3
+    dft2<PK>(a[0], a[1]);
+    dft2<PK>(a[2], a[3]);
+    dft2<PK>(a[4], a[5]);
+    dft2<PK>(a[6], a[7]);
+    // slot 2 k1 + k2 holds X[k1 + 4 k2]
+    float2 t[8];
 #pragma unroll
-  for (int i = 0; i < 8; i++) t[i] = a[i];
+    for (int i = 0; i < 8; i++) t[i] = a[i];
 #pragma unroll
-  for (int k1 = 0; k1 < 4; k1++)
+    for (int k1 = 0; k1 < 4; k1++)
 #pragma unroll
-    for (int k2 = 0; k2 < 2; k2++) a[k1 + 4 * k2] = t[2 * k1 + k2];
-}
-
-template <>
-__device__ __forceinline__ void dft<16>(float2 (&a)[16]) {
+      for (int k2 = 0; k2 < 2; k2++) a[k1 + 4 * k2] = t[2 * k1 + k2];
+  } else {
+    static_assert(R == 16, "radix");
 #pragma unroll
-  for (int n2 = 0; n2 < 4; n2++) dft4(a[n2], a[n2 + 4], a[n2 + 8], a[n2 + 12]);
-  // slot 4 k1 + n2 *= W16^(n2 k1)
-  a[5] = mul_w16<1>(a[5]);
-  a[6] = mul_w16<2>(a[6]);
-  a[7] = mul_w16<3>(a[7]);
-  a[9] = mul_w16<2>(a[9]);
-  a[10] = mul_w16<4>(a[10]);
-  a[11] = mul_w16<6>(a[11]);
-  a[13] = mul_w16<3>(a[13]);
-  a[14] = mul_w16<6>(a[14]);
-  a[15] = mul_w16<9>(a[15]);
+    for (int n2 = 0; n2 < 4; n2++) dft4<PK>(a[n2], a[n2 + 4], a[n2 + 8], a[n2 + 12]);
+    // slot 4 k1 + n2 *= W16^(n2 k1)
+    a[5] = mul_w16<1, PK>(a[5]);
+    a[6] = mul_w16<2, PK>(a[6]);
+    a[7] = mul_w16<3, PK>(a[7]);
+    a[9] = mul_w16<2, PK>(a[9]);
+    a[10] = mul_w16<4, PK>(a[10]);
+    a[11] = mul_w16<6, PK>(a[11]);
+    a[13] = mul_w16<3, PK>(a[13]);
+    a[14] = mul_w16<6, PK>(a[14]);
+    a[15] = mul_w16<9, PK>(a[15]);
 #pragma unroll
-  for (int k1 = 0; k1 < 4; k1++) dft4(a[4 * k1], a[4 * k1 + 1], a[4 * k1 + 2], a[4 * k1 + 3]);
-  float2 t[16];
+    for (int k1 = 0; k1 < 4; k1++) dft4<PK>(a[4 * k1], a[4 * k1 + 1], a[4 * k1 + 2], a[4 * k1 + 3]);
+    float2 t[16];
 #pragma unroll
-  for (int i = 0; i < 16; i++) t[i] = a[i];
+    for (int i = 0; i < 16; i++) t[i] = a[i];
 #pragma unroll
-  for (int k1 = 0; k1 < 4; k1++)
+    for (int k1 = 0; k1 < 4; k1++)
 #pragma unroll
-    for (int k2 = 0; k2 < 4; k2++) a[k1 + 4 * k2] = t[4 * k1 + k2];
+      for (int k2 = 0; k2 < 4; k2++) a[k1 + 4 * k2] = t[4 * k1 + k2];
+  }
 }
 
 __device__ __forceinline__ int padi(int i) { return i + (i >> 4); }
@@ -172,9 +237,9 @@ __device__ __forceinline__ void stage_compute(float2 (&v)[16], int j, const floa
     if constexpr (NS > 1) {
       const int k = vt & (NS - 1);
 #pragma unroll
-      for (int r = 1; r < R; r++) a[r] = cmul(a[r], __ldg(&tw[r * k * (M / (NS * R))]));
+      for (int r = 1; r < R; r++) a[r] = cmul(a[r], __ldg(&tw[tw_stage<R, NS>() + r * NS + k]));
     }
-    dft<R>(a);
+    dft<R, (M > 256)>(a);
 #pragma unroll
     for (int r = 0; r < R; r++) v[u + U * r] = a[r];
   }
@@ -250,13 +315,52 @@ struct LastStage {
 };
 
 
-template <int M, int KIND, bool CG = false>
+// Entries of a line pair's buffer: a pad slot every 16, and a few more so
+// that the pieces of one row that go to adjacent pairs' buffers (staging of
+// column passes: HP = 2048 / M pieces a row) meet different banks.
+__host__ __device__ constexpr int line_buf(int M, int kind) {
+  return M + M / 16 + ((kind == SHIFT_X || kind == ROT_P3) ? 0 : M == 1024 ? 4 : M == 512 ? 2 : M == 256 ? 1 : 0);
+}
+
+// The CTA's lines where they are columns: the 2 LPC adjacent columns from
+// col0 on (row stride RS) of rows [0, N) go row by row, as 16-byte pieces, to
+// the pairs' buffers at `dst` + pair LBUF; a row goes to element `pos(row)`.
+// With 8-byte accesses straight from the pairs' threads a warp touched 32
+// sectors for 256 bytes: rotation pass 2 of 60 frames of n = 1024 1454 -> 1181
+// us, of 500 of n = 256 541 -> 360, shift columns of 777 of n = 128 86 -> 53.
+template <int N, int LPC, int TH, int LBUF, bool CG, class Pos>
+__device__ __forceinline__ void stage_columns(const float *__restrict__ src, size_t RS, float2 *dst, Pos pos) {
+  constexpr int HP = LPC / 2, IT = N * HP / TH;
+  static_assert(HP >= 1 && IT * TH == N * HP, "pieces per thread");
+  constexpr int B = IT < 8 ? IT : 8;   // loads in flight per thread
+#pragma unroll
+  for (int k0 = 0; k0 < IT; k0 += B) {
+    float4 q4[B];
+#pragma unroll
+    for (int k = 0; k < B; k++) {
+      const int i = threadIdx.x + (k0 + k) * TH, row = i / HP, h = i % HP;
+      const float4 *p = reinterpret_cast<const float4 *>(src + (size_t)row * RS + 4 * h);
+      if constexpr (CG) q4[k] = __ldcg(p);
+      else q4[k] = *p;
+    }
+#pragma unroll
+    for (int k = 0; k < B; k++) {
+      const int i = threadIdx.x + (k0 + k) * TH, row = i / HP, h = i % HP;
+      const int e = pos(row);
+      if (e < 0) continue;
+      dst[2 * h * LBUF + padi(e)] = make_float2(q4[k].x, q4[k].y);
+      dst[(2 * h + 1) * LBUF + padi(e)] = make_float2(q4[k].z, q4[k].w);
+    }
+  }
+}
+
+template <int M, int KIND, int TH, bool CG = false>
 __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, int cx, float2 *smem, LineParam *lp,
                                                int *ident_p) {
   constexpr int N = M / 2;
   constexpr int TPL = M / 16;          // threads per line pair
-  constexpr int LPC = 4096 / M;        // line pairs per CTA
-  constexpr int LBUF = M + M / 16;     // padded line buffer, complex entries
+  constexpr int LPC = TH / TPL;        // line pairs per CTA
+  constexpr int LBUF = line_buf(M, KIND);    // padded line buffer, complex entries
   constexpr bool SAME_D = (KIND == SHIFT_X || KIND == SHIFT_Y);
   constexpr int NIN = (KIND == ROT_P3) ? M : N;        // input samples per line
   constexpr int NOUT = (KIND == ROT_P1) ? M : N;       // output samples per line
@@ -269,7 +373,7 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
   const int line0 = 2 * (cx * LPC + p);
   const float *__restrict__ fin = a.in_tab ? a.in_tab[f] : a.in + f * a.in_fstride;
   float *__restrict__ fout = a.out_tab ? a.out_tab[f] : a.out + f * a.out_fstride;
-  const float2 *__restrict__ tw = d_twiddle + tw_off(M);
+  const float2 *__restrict__ tw = d_twiddle;
   float2 *bufA = smem + p * LBUF;
   float2 *bufB = smem + (LPC + p) * LBUF;
   const int q = (KIND == ROT_P1) ? (a.q[f] & 3) : 0;
@@ -319,9 +423,69 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
     return;
   }
 
-  // ---- forward transform, stage 0 straight from global memory ----------
+  // ---- forward transform, stage 0 from global memory, or, where the lines
+  // are columns, from the staged buffer B -------------------------------
+  constexpr bool COLS = (KIND == SHIFT_Y || KIND == ROT_P2);
+  constexpr int RS = (KIND == ROT_P2) ? M : N;     // row stride of a column pass
+  const int col0 = 2 * cx * LPC;
+  float2 *stage = smem + LPC * LBUF;
+  // (M = 128: a warp's four pairs already read 32 bytes of a row; a stride that
+  // suits the staging would make the transforms' exchanges conflict)
+  constexpr bool STAGE = M >= 256;
+  bool staged = COLS && STAGE;
+  if constexpr (COLS && STAGE) {
+    stage_columns<N, LPC, TH, LBUF, CG>(fin + col0, RS, stage, [](int row) { return row; });
+    __syncthreads();
+  }
+  if constexpr (KIND == ROT_P1 && STAGE) {
+    // an odd number of quarter turns: the rows of rot90^q(frame) are columns
+    // of the frame.  (16-byte loads: the allocation-free rotation takes
+    // frames at any float address.)
+    staged = (q & 1) && ((uintptr_t)fin & 15) == 0;
+    if (staged) {
+      if (q == 1) {   // element pos >= 1 of line i is frame[n - pos][i]; element 0 is zero
+        stage_columns<N, LPC, TH, LBUF, CG>(fin + col0, N, stage, [](int row) { return row ? N - row : -1; });
+        if (tid < LPC) stage[tid * LBUF] = make_float2(0.f, 0.f);
+      } else {        // element pos of line i >= 1 is frame[pos][n - i]
+        // the row's columns from n - col0 - 2 LPC on are the lines col0 + 2 LPC
+        // .. col0 + 1, column n - col0 is line col0 (no line for col0 = 0)
+        constexpr int HP = LPC / 2, IT = N * HP / TH;
+        const int cb = N - col0 - 2 * LPC;
+        float *st = reinterpret_cast<float *>(stage);
+        auto put = [&](int u, int row, float x) { st[2 * ((u >> 1) * LBUF + padi(row)) + (u & 1)] = x; };
+#pragma unroll 4
+        for (int k = 0; k < IT; k++) {
+          const int i = tid + k * TH, row = i / HP, h = i % HP;
+          const float *rowp = fin + (size_t)row * N;
+          const float4 *p4 = reinterpret_cast<const float4 *>(rowp + cb + 4 * h);
+          float4 x;
+          if constexpr (CG) x = __ldcg(p4);
+          else x = *p4;
+          const int u = 2 * LPC - 4 * h;   // line of x.x, relative to col0
+          if (h > 0) put(u, row, x.x);
+          put(u - 1, row, x.y);
+          put(u - 2, row, x.z);
+          put(u - 3, row, x.w);
+          if (h == 0) put(0, row, col0 > 0 ? ldf<CG>(rowp + N - col0) : 0.f);
+        }
+      }
+      __syncthreads();
+    }
+  }
   float2 v[16];
-  {
+  if (staged) {
+#pragma unroll
+    for (int m = 0; m < 16; m++) {
+      v[m] = make_float2(0.f, 0.f);
+      if (m * (M / 16) < NIN) {
+        v[m] = bufB[padi(j + m * (M / 16))];
+        if constexpr (KIND == ROT_P1) bad |= !finite_pair(v[m]);
+      }
+    }
+    if constexpr (KIND == ROT_P1) {
+      if (bad) atomicOr(a.status, STATUS_NONFINITE);
+    }
+  } else {
 #pragma unroll
     for (int m = 0; m < 16; m++) {
       const int pos = j + m * (M / 16);
@@ -410,40 +574,58 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
   // ---- store: slot (u, r) -> position vt + r M/R; y = conj(result) -------
   constexpr int RL = LastStage<M>::R;
   constexpr int UL = LastStage<M>::U;
-  {
+  // columns: through the buffer the last stage did not read, then row by row
+  // as 16-byte pieces
+  float2 *ob = (NumStages<M>::value == 2) ? spec : other;
 #pragma unroll
-    for (int u = 0; u < UL; u++) {
+  for (int u = 0; u < UL; u++) {
 #pragma unroll
-      for (int r = 0; r < RL; r++) {
-        const int pos = j + u * (M / 16) + r * (M / RL);
-        if (r * (M / RL) < NOUT) {
-          const float2 y = v[u + UL * r];
-          if constexpr (KIND == SHIFT_Y) {
-            *reinterpret_cast<float2 *>(fout + (size_t)pos * N + line0) = make_float2(y.x, -y.y);
-          } else if constexpr (KIND == ROT_P2) {
-            *reinterpret_cast<float2 *>(fout + (size_t)pos * M + line0) = make_float2(y.x, -y.y);
-          } else {
-            const int rs = (KIND == ROT_P1) ? M : N;
-            fout[(size_t)line0 * rs + pos] = y.x;
-            fout[(size_t)(line0 + 1) * rs + pos] = -y.y;
-          }
+    for (int r = 0; r < RL; r++) {
+      const int pos = j + u * (M / 16) + r * (M / RL);
+      if (r * (M / RL) < NOUT) {
+        const float2 y = v[u + UL * r];
+        if constexpr (COLS && STAGE) {
+          ob[padi(pos)] = make_float2(y.x, -y.y);
+        } else if constexpr (COLS) {
+          *reinterpret_cast<float2 *>(fout + (size_t)pos * RS + line0) = make_float2(y.x, -y.y);
+        } else {
+          const int rs = (KIND == ROT_P1) ? M : N;
+          fout[(size_t)line0 * rs + pos] = y.x;
+          fout[(size_t)(line0 + 1) * rs + pos] = -y.y;
         }
       }
+    }
+  }
+  if constexpr (COLS && STAGE) {
+    __syncthreads();
+    constexpr int HP = LPC / 2;
+    const float2 *o0 = ob - p * LBUF;   // pair 0's
+#pragma unroll 4
+    for (int i = tid; i < N * HP; i += TH) {
+      const int row = i / HP, h = i % HP;
+      const float2 e0 = o0[2 * h * LBUF + padi(row)], e1 = o0[(2 * h + 1) * LBUF + padi(row)];
+      *reinterpret_cast<float4 *>(fout + (size_t)row * RS + col0 + 4 * h) = make_float4(e0.x, e0.y, e1.x, e1.y);
     }
   }
   (void)NLINES;
 }
 
+// Threads per CTA: 256, 512 where 256 would own four columns (16 bytes of a
+// row): column passes of 2048-point lines.
+template <int M, int KIND>
+constexpr int line_threads() { return (M == 2048 && (KIND == SHIFT_Y || KIND == ROT_P2)) ? 512 : 256; }
+
 // One CTA of a line pass: line pairs cx * LPC .. of frame blockIdx.y.
-// Register budget: 3 resident CTAs per SM for lines of up to 256 points, 2
-// for longer ones (measured: 3 is faster on the short lines, slower on the
+// Register budget: 24 resident warps per SM for lines of up to 256 points, 16
+// for longer ones (measured: 24 is faster on the short lines, slower on the
 // 2048-point ones).
 template <int M, int KIND>
-__global__ void __launch_bounds__(256, (M <= 256) ? 3 : 2) line_pass_kernel(const LineArgs a) {
-  extern __shared__ float2 smem[];
-  __shared__ LineParam lp[2 * (4096 / M)];
+__global__ void __launch_bounds__(line_threads<M, KIND>(), ((M <= 256) ? 768 : 512) / line_threads<M, KIND>())
+line_pass_kernel(const LineArgs a) {
+  extern __shared__ __align__(16) float2 smem[];
+  __shared__ LineParam lp[2 * line_threads<M, KIND>() * 16 / M];
   __shared__ int ident_s;
-  line_pass_body<M, KIND>(a, blockIdx.y, blockIdx.x, smem, lp, &ident_s);
+  line_pass_body<M, KIND, line_threads<M, KIND>()>(a, blockIdx.y, blockIdx.x, smem, lp, &ident_s);
 }
 
 // ---------------------------------------------------------------------------
@@ -490,7 +672,7 @@ __device__ __forceinline__ float2 mul_w32(float2 a) {
   else if constexpr (j == 24) return make_float2(-a.y, a.x);
   else {
     constexpr float c = c32(j), s = s32(j);
-    return make_float2(fmaf(a.x, c, a.y * s), fmaf(a.y, c, -a.x * s));
+    return mul_cs<true>(a, c, s);
   }
 }
 
@@ -515,12 +697,12 @@ __device__ __forceinline__ void dft32(float2 (&a)[32]) {
   for (int n2 = 0; n2 < 8; n2++) {
     if constexpr (HALF) {
       const float2 x0 = a[n2], x1 = a[n2 + 8];
-      a[n2] = cadd(x0, x1);
+      a[n2] = padd(x0, x1);
       a[n2 + 8] = make_float2(x0.x + x1.y, x0.y - x1.x);    // x0 - i x1
-      a[n2 + 16] = csub(x0, x1);
+      a[n2 + 16] = psub(x0, x1);
       a[n2 + 24] = make_float2(x0.x - x1.y, x0.y + x1.x);   // x0 + i x1
     } else {
-      dft4(a[n2], a[n2 + 8], a[n2 + 16], a[n2 + 24]);
+      dft4<true>(a[n2], a[n2 + 8], a[n2 + 16], a[n2 + 24]);
     }
   }
   w32_row<1>(a);
@@ -532,7 +714,7 @@ __device__ __forceinline__ void dft32(float2 (&a)[32]) {
     float2 b[8];
 #pragma unroll
     for (int n2 = 0; n2 < 8; n2++) b[n2] = a[8 * k1 + n2];
-    dft<8>(b);
+    dft<8, true>(b);
 #pragma unroll
     for (int k2 = 0; k2 < 8; k2++) t[k1 + 4 * k2] = b[k2];
   }
@@ -599,11 +781,12 @@ __device__ __forceinline__ void w32_filter(float2 (&v)[32], int lane, float2 *bu
     // lines a and b shifted by their own amounts.  Bins k and M - k share the
     // separated spectra (A_{M-k} = conj A_k, B_{M-k} = conj B_k) and the
     // phasors (H_{-k} = conj H_k), so each lane computes its bins k < M/2
-    // (r < 16) and hands V_{M-k} to the lane that holds bin M - k; lane 0
-    // computes its own bins 0 and M/2 (each its own partner).
-#pragma unroll
-    for (int r = 0; r < 32; r++) buf[pad32(lane + 32 * r)] = v[r];
-    __syncwarp();
+    // (r < 16), with Z_{M-k} from the lane that holds bin M - k = (32 - lane)
+    // + 32 (31 - r), and hands V_{M-k} back.  Shuffles: 64 wavefronts a pair
+    // where writing the spectrum out and reading partner by partner took 160
+    // (800 frames: pass 1 862 -> 839 us, pass 3 649 -> 620).  Lane 0's partners, bins 1024 - 32 r, are its own
+    // registers 32 - r; bins 0 and M/2 are their own partners.
+    const int partner = (32 - lane) & 31;
     const float2 sb = phase_at(lb, 32);
     float2 ha, hb;
 #pragma unroll
@@ -617,15 +800,20 @@ __device__ __forceinline__ void w32_filter(float2 (&v)[32], int lane, float2 *bu
         ha = cmul(ha, sa);
         hb = cmul(hb, sb);
       }
-      // twice the spectra of lines a and b; location M - k is read and
-      // written by this lane only
-      const int jm = pad32((M - k) & (M - 1));
-      const float2 z = v[r], zm = buf[jm];
+      // twice the spectra of lines a and b
+      const float2 own = v[(32 - r) & 31];
+      float2 zm = make_float2(__shfl_sync(0xffffffffu, v[31 - r].x, partner),
+                              __shfl_sync(0xffffffffu, v[31 - r].y, partner));
+      zm = lane == 0 ? own : zm;
+      const float2 z = v[r];
       const float2 A = make_float2(z.x + zm.x, z.y - zm.y);
       const float2 B = make_float2(z.y + zm.y, zm.x - z.x);
       const float2 P = cmul(A, ha), Q = cmul(B, hb);
       v[r] = make_float2(P.x - Q.y, -(P.y + Q.x));                 // conj(V_k) / m
-      if (r > 0 || lane > 0) buf[jm] = make_float2(P.x + Q.y, P.y - Q.x);   // conj(V_{M-k}) / m
+      const float2 w = make_float2(P.x + Q.y, P.y - Q.x);          // conj(V_{M-k}) / m
+      const float2 back = make_float2(__shfl_sync(0xffffffffu, w.x, partner), __shfl_sync(0xffffffffu, w.y, partner));
+      v[31 - r] = lane == 0 ? v[31 - r] : back;
+      if (r > 0) v[32 - r] = lane == 0 ? w : v[32 - r];
     }
     if (lane == 0) {   // Nyquist bin M/2: v[16] holds it, its own partner
       const float2 z = v[16];
@@ -634,12 +822,7 @@ __device__ __forceinline__ void w32_filter(float2 (&v)[32], int lane, float2 *bu
       const float2 P = cmul(A, make_float2(la.cnyq * sc, 0.f)), Q = cmul(B, make_float2(lb.cnyq * sc, 0.f));
       v[16] = make_float2(P.x - Q.y, -(P.y + Q.x));
     }
-    __syncwarp();
-#pragma unroll
-    for (int r = 16; r < 32; r++)
-      if (r > 16 || lane > 0) v[r] = buf[pad32(lane + 32 * r)];
   }
-  __syncwarp();
 
   // ---- inverse: the same stages on conj(V)/m; y = conj(result) ------------
   fft1024_warp(v, lane, buf, tw);
@@ -654,7 +837,12 @@ __device__ __forceinline__ void w32_filter(float2 (&v)[32], int lane, float2 *bu
 // than 12 for every kind).
 template <int KIND>
 constexpr int w32_ppc() { return (KIND == ROT_P2 || KIND == ROT_P1) ? 8 : 4; }
-constexpr size_t w32_smem_bytes(int ppc) { return (size_t)ppc * (1024 + 1024 / 32) * sizeof(float2); }
+// Entries of a warp's exchange buffer: a pad slot every 32, and a few more so
+// that the pieces of one row that go to adjacent pairs' buffers (the staging
+// of columns: ppc / 2 pieces a row) meet different banks (four-way conflicts
+// without them: 800 frames, pass 2 1888 -> 1693 us, shift columns 762 -> 735).
+constexpr int w32_buf(int ppc) { return 1024 + 32 + (ppc == 8 ? 2 : 4); }
+constexpr size_t w32_smem_bytes(int ppc) { return (size_t)ppc * w32_buf(ppc) * sizeof(float2); }
 
 template <int KIND>
 __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) line_pass_w32(const LineArgs a) {
@@ -663,7 +851,7 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
   constexpr int NIN = (KIND == ROT_P3) ? M : N;
   constexpr int NOUT = (KIND == ROT_P1) ? M : N;
   extern __shared__ float2 w32_smem[];
-  float2 (*sbuf)[M + M / 32] = reinterpret_cast<float2 (*)[M + M / 32]>(w32_smem);   // [PPC][M + M/32]
+  float2 (*sbuf)[w32_buf(PPC)] = reinterpret_cast<float2 (*)[w32_buf(PPC)]>(w32_smem);
   __shared__ LineParam lp[PPC][2];
   __shared__ int ident_s;
 
@@ -948,11 +1136,11 @@ __device__ __forceinline__ void batch_pass(const BatchFrame &fr, int cx, int *st
   // shift passes read only the input (or lines only their own CTA wrote).
   constexpr bool CG = (KIND == ROT_P1 || KIND == ROT_P2 || KIND == ROT_P3);
   switch (fr.n) {
-    case 64: line_pass_body<128, KIND, CG>(la, 0, cx, smem, lp, ident); break;
-    case 128: line_pass_body<256, KIND, CG>(la, 0, cx, smem, lp, ident); break;
-    case 256: line_pass_body<512, KIND, CG>(la, 0, cx, smem, lp, ident); break;
-    case 512: line_pass_body<1024, KIND, CG>(la, 0, cx, smem, lp, ident); break;
-    default: line_pass_body<2048, KIND, CG>(la, 0, cx, smem, lp, ident); break;
+    case 64: line_pass_body<128, KIND, 256, CG>(la, 0, cx, smem, lp, ident); break;
+    case 128: line_pass_body<256, KIND, 256, CG>(la, 0, cx, smem, lp, ident); break;
+    case 256: line_pass_body<512, KIND, 256, CG>(la, 0, cx, smem, lp, ident); break;
+    case 512: line_pass_body<1024, KIND, 256, CG>(la, 0, cx, smem, lp, ident); break;
+    default: line_pass_body<2048, KIND, 256, CG>(la, 0, cx, smem, lp, ident); break;
   }
 }
 
@@ -973,7 +1161,7 @@ __device__ __forceinline__ bool wait_at_least(const int *ctr, int target, long l
 constexpr int BATCH_GRAB = 4;
 
 __global__ void __launch_bounds__(256, 2) batch_persistent_kernel(const BatchArgs b) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   __shared__ LineParam lp[2 * 32];
   __shared__ int ident_s;
   __shared__ int grab_s[2];
@@ -1024,19 +1212,21 @@ __global__ void __launch_bounds__(256, 2) batch_persistent_kernel(const BatchArg
   }
 }
 
-template <int M>
-size_t line_smem_bytes() {
-  constexpr int LPC = 4096 / M;
-  constexpr int LBUF = M + M / 16;
-  return (size_t)2 * LPC * LBUF * sizeof(float2);
+// two buffers per line pair
+constexpr size_t line_smem_bytes(int M, int threads, int kind) {
+  return (size_t)2 * (threads * 16 / M) * line_buf(M, kind) * sizeof(float2);
 }
+constexpr size_t kBatchSmem = line_smem_bytes(256, 256, ROT_P2);   // the largest over the line lengths
+static_assert(kBatchSmem >= line_smem_bytes(128, 256, ROT_P2) && kBatchSmem >= line_smem_bytes(512, 256, ROT_P2) &&
+              kBatchSmem >= line_smem_bytes(1024, 256, ROT_P2) && kBatchSmem >= line_smem_bytes(2048, 256, ROT_P2), "largest buffer");
 
 template <int M, int KIND>
 cudaError_t launch_one(const LineArgs &a, long long n_frames, cudaStream_t st) {
   constexpr int N = M / 2;
-  constexpr int LPC = 4096 / M;
+  constexpr int TH = line_threads<M, KIND>();
+  constexpr int LPC = TH * 16 / M;
   constexpr int NLINES = (KIND == ROT_P2) ? M : N;
-  const size_t smem = line_smem_bytes<M>();   // limit raised by geom_init_device
+  constexpr size_t smem = line_smem_bytes(M, TH, KIND);   // limit raised by geom_init_device
   for (long long f0 = 0; f0 < n_frames; f0 += 65535) {
     const long long nf = (n_frames - f0 < 65535) ? (n_frames - f0) : 65535;
     LineArgs b = a;
@@ -1049,7 +1239,7 @@ cudaError_t launch_one(const LineArgs &a, long long n_frames, cudaStream_t st) {
     b.out_tab = a.out_tab ? a.out_tab + f0 : nullptr;
     b.lp_tab = a.lp_tab ? reinterpret_cast<const LineParam *>(a.lp_tab) + f0 * a.lp_lines : nullptr;
     dim3 grid(NLINES / (2 * LPC), (unsigned)nf);
-    line_pass_kernel<M, KIND><<<grid, 256, smem, st>>>(b);
+    line_pass_kernel<M, KIND><<<grid, TH, smem, st>>>(b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1072,13 +1262,15 @@ cudaError_t launch_m(LineKind kind, const LineArgs &a, long long n_frames, cudaS
 // length M (done once per device at set-up, outside any stream capture).
 template <int M>
 bool configure_m() {
-  const int smem = (int)line_smem_bytes<M>();
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  return cudaFuncSetAttribute(line_pass_kernel<M, SHIFT_X>, at, smem) == cudaSuccess &&
-         cudaFuncSetAttribute(line_pass_kernel<M, SHIFT_Y>, at, smem) == cudaSuccess &&
-         cudaFuncSetAttribute(line_pass_kernel<M, ROT_P1>, at, smem) == cudaSuccess &&
-         cudaFuncSetAttribute(line_pass_kernel<M, ROT_P2>, at, smem) == cudaSuccess &&
-         cudaFuncSetAttribute(line_pass_kernel<M, ROT_P3>, at, smem) == cudaSuccess;
+  auto set = [&](auto kernel, int threads, int kind) {
+    return cudaFuncSetAttribute(kernel, at, (int)line_smem_bytes(M, threads, kind)) == cudaSuccess;
+  };
+  return set(line_pass_kernel<M, SHIFT_X>, line_threads<M, SHIFT_X>(), SHIFT_X) &&
+         set(line_pass_kernel<M, SHIFT_Y>, line_threads<M, SHIFT_Y>(), SHIFT_Y) &&
+         set(line_pass_kernel<M, ROT_P1>, line_threads<M, ROT_P1>(), ROT_P1) &&
+         set(line_pass_kernel<M, ROT_P2>, line_threads<M, ROT_P2>(), ROT_P2) &&
+         set(line_pass_kernel<M, ROT_P3>, line_threads<M, ROT_P3>(), ROT_P3);
 }
 
 }  // namespace
@@ -1135,27 +1327,30 @@ int geom_init_device() {
   // the persistent batch kernel is launched inside stream capture: set its
   // shared-memory limit here, per device, outside any capture
   if (cudaFuncSetAttribute(batch_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)line_smem_bytes<1024>()) != cudaSuccess)
+                           (int)kBatchSmem) != cudaSuccess)
     return -1;
-  static float2 host[kTwTotal];
+  static float2 host[kTwTotal], rl[32 * 32];
   static bool filled = false;
   if (!filled) {
-    for (int m = 128; m <= 2048; m *= 2)
-      for (int e = 0; e < m; e++) {
-        const double ang = 2.0 * 3.14159265358979323846 * (double)e / (double)m;
-        host[tw_off(m) + e] = make_float2((float)cos(ang), (float)-sin(ang));
-      }
+    auto fill = [](float2 *t, int rows, int cols, int m) {   // [r][k] = W_m^(r k)
+      for (int r = 0; r < rows; r++)
+        for (int k = 0; k < cols; k++) {
+          const double ang = 2.0 * 3.14159265358979323846 * (double)(r * k) / (double)m;
+          t[r * cols + k] = make_float2((float)cos(ang), (float)-sin(ang));
+        }
+    };
+    fill(host + kTwS1, 16, 16, 256);
+    fill(host + kTwS1b, 8, 16, 128);
+    for (int m = 512; m <= 2048; m *= 2) fill(host + kTwS2 + m - 512, m / 256, 256, m);
+    fill(rl, 32, 32, 1024);
     filled = true;
   }
-  static float2 rl[32 * 32];
-  for (int r = 0; r < 32; r++)
-    for (int l = 0; l < 32; l++) rl[r * 32 + l] = host[tw_off(1024) + r * l];
   if (cudaMemcpyToSymbol(d_tw1024_rl, rl, sizeof(rl)) != cudaSuccess) return -1;
   return cudaMemcpyToSymbol(d_twiddle, host, sizeof(host)) == cudaSuccess ? 0 : -1;
 }
 
 cudaError_t launch_batch_persistent(const BatchArgs &b, int ctas_per_sm, cudaStream_t st) {
-  const size_t smem = line_smem_bytes<1024>();   // the same for every line length
+  const size_t smem = kBatchSmem;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
