@@ -10,17 +10,23 @@
 //    packed (total-order key of the value, ~index): the largest value wins,
 //    the smallest index on a tie.  A non-finite value sets the word to all
 //    ones (no finite value packs to it) and the status flag.
-//  * register_fit_kernel: one warp per frame.  The box of half-size R around
-//    the seed and its 8-connected flood fill in shared memory (sweeps until
-//    none changes: the fixpoint is the connected component whatever the
-//    order of the updates), FP64 patch sums, then the fit window in the same
-//    shared buffer and the Levenberg-Marquardt loop.  Every sum is a
-//    butterfly (xor) shuffle reduction, which leaves the bit-identical sum in
-//    every lane (each level adds the same two operands, commuted), so every
-//    lane solves the same damped 6 x 6 system and takes the same decisions:
-//    no broadcast, no block barrier, and several frames per SM keep the FP64
-//    pipe busy.  Start values, damping schedule and stopping rules are those
-//    of the FP64 oracle.
+//  * register_fit_kernel: one block of FIT_WARPS warps per frame.  The box of
+//    half-size R around the seed and its 8-connected flood fill in shared
+//    memory (sweeps until none changes: the fixpoint is the connected
+//    component whatever the order of the updates), FP64 patch sums, then the
+//    fit window in the same shared buffer and the Levenberg-Marquardt loop.
+//    Warp 0 holds the parameters, solves the damped 6 x 6 system and takes
+//    the decisions; the model and its derivatives are evaluated by every
+//    warp, a pixel per thread, into shared memory, and the 28 sums of the
+//    normal equations are then taken seven to a warp.  Each sum is taken in
+//    one fixed order (32 strided partials, then a butterfly over them).
+//    Start values, damping schedule and stopping rules are those of the FP64
+//    oracle.
+//    Bound: the FP64 pipe (a warp instruction takes it 16 cycles; 14,500 of
+//    them per fitted frame) and, below a few frames per SM, the latency of
+//    the chain evaluate - sum - solve.  With a frame on one warp that chain
+//    was all there was; measured calls, then -> now, same bits: one frame
+//    612 -> 315 us, 400 of 256 x 256 1259 -> 774, 1600 2084 -> 1849.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -33,7 +39,12 @@ namespace {
 constexpr int ARG_THREADS = 256;
 constexpr int ARG_VEC = 8;                                   // float4 loads per thread per chunk
 constexpr long long REG_CHUNK = (long long)ARG_THREADS * ARG_VEC * 4;   // pixels per block
-constexpr int FIT_WARPS = 1;   // one warp (frame) per block: small batches spread over all SMs
+// Warps per block (frame): the sums take four.  With three blocks per SM 400
+// frames take 779 us; two 887, one 1118, four 781, two of eight warps 872.
+constexpr int FIT_WARPS = 4;
+constexpr int FIT_THREADS = 32 * FIT_WARPS;
+constexpr int FIT_TILE = 512;  // window pixels whose model values are in shared memory at a time
+constexpr int FIT_Z = 6;       // values per pixel there: dI/dI0, dx0, dy0, dalpha, dbeta and the residual
 constexpr double REG_PI = 3.14159265358979323846;
 constexpr unsigned long long KEY_NONFINITE = ~0ull;
 
@@ -136,12 +147,6 @@ __device__ __forceinline__ double warp_sum(double x) {
   return x;
 }
 
-__device__ __forceinline__ float warp_sum32(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
-
 __device__ __forceinline__ float warp_min(float x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
@@ -213,50 +218,190 @@ __device__ bool chol6(const double *A, const double *b, double *x) {
   return true;
 }
 
-// One pass over the window at the parameters k: the squared error of the
-// model and the normal equations of its analytic Jacobian (J^T J lower
-// triangle in ne[0..21), J^T r in ne[21..27)), lane partials then warp sums
-// (every lane ends with the same values).  The oracle takes the two in
-// separate passes; one pass serves both here because the normal equations
-// of an accepted trial point are those of the next iteration.
-__device__ __forceinline__ double window_pass(const MoffatConst &k, const float *win, int WH, int WW, int wr0,
-                                              int wc0, int lane, double *ne) {
-  double cost = 0.0;
+// What the warps of a block share besides the window and the model values.
+struct FitShared {
+  double kc[11];      // MoffatConst of the parameters to evaluate
+  float kf[11];       // the same in FP32
+  double ne[28];      // the last evaluation's sums: J^T J lower triangle, J^T r, the squared error
+  double ne_cur[28];  // those of the current parameters
+  double patch[4];    // patch size, value sum and first moments
+  int mode;           // what to evaluate next (EVAL_*)
+  int touch;          // the patch touches the box's inner border
+  long long frame;
+};
+enum { EVAL_DONE = 0, EVAL_F32 = 1, EVAL_F64 = 2 };
+
+// Barrier of all the block's warps, for the places where warp 0 and the
+// others wait at different instructions.
+__device__ __forceinline__ void fit_sync() { asm volatile("bar.sync 1, %0;" ::"n"(FIT_THREADS) : "memory"); }
+
+// Model values of one pixel at the parameters k: derivatives by I0, x0, y0,
+// alpha, beta (the one by Bg is 1) and the residual.  Where a sum of two
+// products leaves open which of them is rounded, the fused form is written
+// out: alpha and beta are so correlated that a last bit here moves them by
+// 1e-8, so the bits must not depend on how the compiler orders the code.
+__device__ __forceinline__ void moffat_pixel(const MoffatConst &k, int col, int row, float val, double (&z)[FIT_Z]) {
+  const double dx = (double)col - k.x0, dy = (double)row - k.y0;
+  const double rho2 = fma(dy, dy, dx * dx);
+  const double u = 1.0 + rho2 * k.ia2;
+  const double lu = log(u);
+  const double P = exp(-k.beta * lu);
+  // 1 / u: the FP32 reciprocal refined by two Newton steps r <- r (2 - u r)
+  // (relative error 1e-7 -> 1e-14 -> below FP64 rounding; u >= 1)
+  double ru = (double)__frcp_rn((float)u);
+  ru = ru * (2.0 - u * ru);
+  ru = ru * (2.0 - u * ru);
+  const double Pu = P * ru;
+  z[5] = k.A * P + k.bg - (double)val;
+  z[0] = k.c0 * P;
+  z[1] = k.c1 * Pu * dx;
+  z[2] = k.c1 * Pu * dy;
+  z[3] = fma(k.c4 * rho2, Pu, k.c3 * P);
+  z[4] = fma(k.c5, P, -(k.A * lu * P));
+}
+
+// The same in FP32: on GB300 the FP32 pipe is 64 times the FP64 one, and the
+// first iterations only need to come close.
+struct MoffatConst32 {
+  float x0, y0, beta, bg, ia2, A, c0, c1, c3, c4, c5;
+};
+
+__device__ __forceinline__ void moffat_pixel(const MoffatConst32 &k, int col, int row, float val, float (&z)[FIT_Z]) {
+  const float dx = (float)col - k.x0, dy = (float)row - k.y0;
+  const float rho2 = fmaf(dy, dy, dx * dx);
+  const float u = 1.0f + rho2 * k.ia2;
+  const float l2 = log2f(u);
+  const float P = exp2f(-k.beta * l2);
+  const float Pu = P / u;
+  z[5] = k.A * P + k.bg - val;
+  z[0] = k.c0 * P;
+  z[1] = k.c1 * Pu * dx;
+  z[2] = k.c1 * Pu * dy;
+  z[3] = fmaf(k.c3, P, k.c4 * rho2 * Pu);
+  z[4] = fmaf(k.c5, P, -(k.A * (l2 * 0.69314718056f) * P));
+}
+
+// The seven sums of group G over the tile's pixels lane, lane + 32, ... (the
+// 28 products of derivatives and residual; the derivative by Bg is 1):
+//   0  residual x (five derivatives, 1, residual)
+//   1  1 x (five derivatives, 1); dI0 dI0
+//   2  dbeta x (five derivatives); dx0 x (dI0, dx0)
+//   3  dalpha x (dI0, dx0, dy0, dalpha); dy0 x (dI0, dx0, dy0)
+template <int G, class R>
+__device__ __forceinline__ void group_sums(const R *z, int count, int lane, R (&acc)[8]) {
+#pragma unroll 2
+  for (int i = lane; i < count; i += 32) {
+    R v[FIT_Z];
 #pragma unroll
-  for (int q = 0; q < 27; q++) ne[q] = 0.0;
-  for (int i = lane; i < WH * WW; i += 32) {
-    const int r = i / WW, c = i - r * WW;
-    const double dx = (double)(c + wc0) - k.x0, dy = (double)(r + wr0) - k.y0;
-    const double rho2 = dx * dx + dy * dy;
-    const double u = 1.0 + rho2 * k.ia2;
-    const double lu = log(u);
-    const double P = exp(-k.beta * lu);
-    // 1 / u: the FP32 reciprocal refined by two Newton steps r <- r (2 - u r)
-    // (relative error 1e-7 -> 1e-14 -> below FP64 rounding; u >= 1)
-    double ru = (double)__frcp_rn((float)u);
-    ru = ru * (2.0 - u * ru);
-    ru = ru * (2.0 - u * ru);
-    const double Pu = P * ru;
-    const double e = k.A * P + k.bg - (double)win[i];
-    double g[6];
-    g[0] = k.c0 * P;
-    g[1] = k.c1 * Pu * dx;
-    g[2] = k.c1 * Pu * dy;
-    g[3] = k.c3 * P + k.c4 * rho2 * Pu;
-    g[4] = k.c5 * P - k.A * lu * P;
-    g[5] = 1.0;
-    cost += e * e;
-    int q = 0;
+    for (int c = 0; c < FIT_Z; c++) v[c] = z[c * FIT_TILE + i];   // those unused are dropped
+    if constexpr (G == 0) {
 #pragma unroll
-    for (int ii = 0; ii < 6; ii++)
+      for (int c = 0; c < 5; c++) acc[c] += v[c] * v[5];
+      acc[5] += v[5];
+      acc[6] += v[5] * v[5];
+    } else if constexpr (G == 1) {
 #pragma unroll
-      for (int jj = 0; jj <= ii; jj++) ne[q++] += g[ii] * g[jj];
+      for (int c = 0; c < 5; c++) acc[c] += v[c];
+      acc[5] += (R)1;
+      acc[6] += v[0] * v[0];
+    } else if constexpr (G == 2) {
 #pragma unroll
-    for (int ii = 0; ii < 6; ii++) ne[21 + ii] += g[ii] * e;
+      for (int c = 0; c < 5; c++) acc[c] += v[4] * v[c];
+      acc[5] += v[1] * v[0];
+      acc[6] += v[1] * v[1];
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; c++) acc[c] += v[3] * v[c];
+#pragma unroll
+      for (int c = 0; c < 3; c++) acc[4 + c] += v[2] * v[c];
+    }
   }
+}
+
+// Place of sum j of group G among the 28 (row i of the triangle starts at
+// i (i + 1) / 2).
+template <int G>
+__device__ __forceinline__ int group_place(int j) {
+  if constexpr (G == 0) return 21 + j;
+  else if constexpr (G == 1) return j < 6 ? 15 + j : 0;
+  else if constexpr (G == 2) return j < 5 ? 10 + j : j - 4;
+  else return j < 4 ? 6 + j : j - 1;
+}
+
+// Butterfly sums of acc[0..8) over the warp, halving what a lane holds at
+// each of the first three levels (9 additions for 8 sums instead of 40; every
+// addition adds the two operands that the full butterfly adds, so the bits
+// are those of eight full ones): acc[0] ends as the sum of slot
+// 4 (lane & 16) / 16 + 2 (lane & 8) / 8 + (lane & 4) / 4.
+template <class R>
+__device__ __forceinline__ void butterfly8(R (&acc)[8], int lane) {
 #pragma unroll
-  for (int q = 0; q < 27; q++) ne[q] = warp_sum(ne[q]);
-  return warp_sum(cost);
+  for (int o = 16, h = 4; o >= 4; o >>= 1, h >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < h; k++) {
+      const R send = up ? acc[k] : acc[k + h], keep = up ? acc[k + h] : acc[k];
+      acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+}
+
+template <int G, class R>
+__device__ __forceinline__ void group_finish(R (&acc)[8], int lane, double *ne) {
+  butterfly8(acc, lane);
+  const int j = (lane >> 2) & 7, slot = ((j & 4) ? 4 : 0) + ((j & 2) ? 2 : 0) + (j & 1);
+  if ((lane & 3) == 0 && slot < 7) ne[group_place<G>(slot)] = (double)acc[0];
+}
+
+// One pass over the window at the shared parameters, by every warp of the
+// block: the squared error of the model and the normal equations of its
+// analytic Jacobian, in s.ne when the closing barrier has passed.  The oracle
+// takes the two in separate passes; one pass serves both here because the
+// normal equations of an accepted trial point are those of the next
+// iteration.
+template <class R, class K>
+__device__ __forceinline__ void window_pass(const K &k, FitShared &s, R *z, const float *win, int WH, int WW, int wr0,
+                                            int wc0) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int np = WH * WW;
+  R acc[8] = {};
+  for (int t0 = 0; t0 < np; t0 += FIT_TILE) {
+    const int count = min(FIT_TILE, np - t0);
+    if (t0 > 0) fit_sync();   // the sums have read the tile before
+    for (int i = threadIdx.x; i < count; i += FIT_THREADS) {
+      const int r = (t0 + i) / WW, c = t0 + i - r * WW;
+      R v[FIT_Z];
+      moffat_pixel(k, c + wc0, r + wr0, win[t0 + i], v);
+#pragma unroll
+      for (int q = 0; q < FIT_Z; q++) z[q * FIT_TILE + i] = v[q];
+    }
+    fit_sync();
+    if (wid == 0) group_sums<0>(z, count, lane, acc);
+    else if (wid == 1) group_sums<1>(z, count, lane, acc);
+    else if (wid == 2) group_sums<2>(z, count, lane, acc);
+    else if (wid == 3) group_sums<3>(z, count, lane, acc);
+  }
+  if (wid == 0) group_finish<0>(acc, lane, s.ne);
+  else if (wid == 1) group_finish<1>(acc, lane, s.ne);
+  else if (wid == 2) group_finish<2>(acc, lane, s.ne);
+  else if (wid == 3) group_finish<3>(acc, lane, s.ne);
+  fit_sync();
+}
+
+// The parameters' quotients from shared memory, then the pass.
+__device__ __forceinline__ void window_pass_shared(int mode, FitShared &s, unsigned char *zb, const float *win, int WH,
+                                                   int WW, int wr0, int wc0) {
+  if (mode == EVAL_F32) {
+    const MoffatConst32 k = {s.kf[0], s.kf[1], s.kf[2], s.kf[3], s.kf[4], s.kf[5],
+                             s.kf[6], s.kf[7], s.kf[8], s.kf[9], s.kf[10]};
+    window_pass<float>(k, s, reinterpret_cast<float *>(zb), win, WH, WW, wr0, wc0);
+  } else {
+    const MoffatConst k = {s.kc[0], s.kc[1], s.kc[2], s.kc[3], s.kc[4], s.kc[5],
+                           s.kc[6], s.kc[7], s.kc[8], s.kc[9], s.kc[10]};
+    window_pass<double>(k, s, reinterpret_cast<double *>(zb), win, WH, WW, wr0, wc0);
+  }
 }
 
 // The damped step of the FP32 phase: the normal equations scaled by D =
@@ -310,65 +455,27 @@ __device__ bool step32(const double *ne, double lambda, double *d) {
   return true;
 }
 
-// The same quotients in FP32, for the first (FP32) phase of the fit.
-struct MoffatConst32 {
-  float x0, y0, beta, bg, ia2, A, c0, c1, c3, c4, c5;
-};
-
-__device__ __forceinline__ MoffatConst32 moffat_const32(const double *p) {
+// Evaluation at the parameters p, called by warp 0: hands the quotients to
+// the block and takes part in the pass.  Returns the squared error (the other
+// sums are in s.ne).
+template <bool F32>
+__device__ __forceinline__ double evaluate(const double *p, FitShared &s, unsigned char *zb, const float *win, int WH,
+                                           int WW, int wr0, int wc0) {
+  const int lane = threadIdx.x & 31;
   const MoffatConst k = moffat_const(p);
-  MoffatConst32 f;
-  f.x0 = (float)k.x0;
-  f.y0 = (float)k.y0;
-  f.beta = (float)k.beta;
-  f.bg = (float)k.bg;
-  f.ia2 = (float)k.ia2;
-  f.A = (float)k.A;
-  f.c0 = (float)k.c0;
-  f.c1 = (float)k.c1;
-  f.c3 = (float)k.c3;
-  f.c4 = (float)k.c4;
-  f.c5 = (float)k.c5;
-  return f;
-}
-
-// window_pass with the per-pixel model, derivatives, lane partials and warp
-// sums in FP32: on GB300 the FP32 pipe is 64 times the FP64 one, and the
-// first iterations only need to come close.
-__device__ __forceinline__ double window_pass32(const MoffatConst32 &k, const float *win, int WH, int WW, int wr0,
-                                                int wc0, int lane, double *ne) {
-  float cost = 0.0f, a[27];
+  __syncwarp();   // every lane has read the last evaluation's sums
+  if (lane == 0) {
+    const double v[11] = {k.x0, k.y0, k.beta, k.bg, k.ia2, k.A, k.c0, k.c1, k.c3, k.c4, k.c5};
 #pragma unroll
-  for (int q = 0; q < 27; q++) a[q] = 0.0f;
-  for (int i = lane; i < WH * WW; i += 32) {
-    const int r = i / WW, c = i - r * WW;
-    const float dx = (float)(c + wc0) - k.x0, dy = (float)(r + wr0) - k.y0;
-    const float rho2 = dx * dx + dy * dy;
-    const float u = 1.0f + rho2 * k.ia2;
-    const float l2 = log2f(u);
-    const float P = exp2f(-k.beta * l2);
-    const float Pu = P / u;
-    const float e = k.A * P + k.bg - win[i];
-    float g[6];
-    g[0] = k.c0 * P;
-    g[1] = k.c1 * Pu * dx;
-    g[2] = k.c1 * Pu * dy;
-    g[3] = k.c3 * P + k.c4 * rho2 * Pu;
-    g[4] = k.c5 * P - k.A * (l2 * 0.69314718056f) * P;
-    g[5] = 1.0f;
-    cost += e * e;
-    int q = 0;
-#pragma unroll
-    for (int ii = 0; ii < 6; ii++)
-#pragma unroll
-      for (int jj = 0; jj <= ii; jj++) a[q++] += g[ii] * g[jj];
-#pragma unroll
-    for (int ii = 0; ii < 6; ii++) a[21 + ii] += g[ii] * e;
+    for (int q = 0; q < 11; q++) {
+      if constexpr (F32) s.kf[q] = (float)v[q];
+      else s.kc[q] = v[q];
+    }
+    s.mode = F32 ? EVAL_F32 : EVAL_F64;
   }
-  // FP32 butterflies (each lane ends with the same bits), widened at the end
-#pragma unroll
-  for (int q = 0; q < 27; q++) ne[q] = (double)warp_sum32(a[q]);
-  return (double)warp_sum32(cost);
+  fit_sync();
+  window_pass_shared(F32 ? EVAL_F32 : EVAL_F64, s, zb, win, WH, WW, wr0, wc0);
+  return s.ne[27];
 }
 
 // Levenberg-Marquardt iterations from p (the oracle's steps: damping lambda
@@ -378,17 +485,13 @@ __device__ __forceinline__ double window_pass32(const MoffatConst32 &k, const fl
 // of it, when no try lowers it, or after 200 iterations).  F32 selects the
 // FP32 evaluation.  Returns the iterations made; p and cost are updated.
 template <bool F32>
-__device__ __forceinline__ int lm_loop(double (&p)[6], double &cost, double *ne_cur, double lam_floor,
-                                       double stop_rel, const float *buf, int WH, int WW, int wr0, int wc0,
-                                       int lane) {
-  double ne[27];
-  cost = F32 ? window_pass32(moffat_const32(p), buf, WH, WW, wr0, wc0, lane, ne)
-             : window_pass(moffat_const(p), buf, WH, WW, wr0, wc0, lane, ne);
-  // ne_cur: the normal equations at p (identical in every lane: lane q keeps q)
-  __syncwarp();
-#pragma unroll
-  for (int q = 0; q < 27; q++)
-    if (lane == q) ne_cur[q] = ne[q];
+__device__ __forceinline__ int lm_loop(double (&p)[6], double &cost, double lam_floor, double stop_rel, FitShared &s,
+                                       unsigned char *zb, const float *buf, int WH, int WW, int wr0, int wc0) {
+  const int lane = threadIdx.x & 31;
+  const double *ne_cur = s.ne_cur;
+  cost = evaluate<F32>(p, s, zb, buf, WH, WW, wr0, wc0);
+  // the normal equations at p
+  if (lane < 27) s.ne_cur[lane] = s.ne[lane];
   __syncwarp();
   double lambda = 1e-3;
   int it;
@@ -429,15 +532,12 @@ __device__ __forceinline__ int lm_loop(double (&p)[6], double &cost, double *ne_
         lambda *= 10.0;
         continue;
       }
-      newcost = F32 ? window_pass32(moffat_const32(q), buf, WH, WW, wr0, wc0, lane, ne)
-                    : window_pass(moffat_const(q), buf, WH, WW, wr0, wc0, lane, ne);
+      newcost = evaluate<F32>(q, s, zb, buf, WH, WW, wr0, wc0);
       if (newcost < cost) {
 #pragma unroll
         for (int ii = 0; ii < 6; ii++) p[ii] = q[ii];
         __syncwarp();   // every lane has read ne_cur
-#pragma unroll
-        for (int qq = 0; qq < 27; qq++)
-          if (lane == qq) ne_cur[qq] = ne[qq];
+        if (lane < 27) s.ne_cur[lane] = s.ne[lane];
         __syncwarp();
         lambda = fmax(lambda / 10.0, lam_floor);
         accepted = true;
@@ -456,15 +556,18 @@ __device__ __forceinline__ int lm_loop(double (&p)[6], double &cost, double *ne_
   return it;
 }
 
-// One frame on one warp: seed from the argmax word, patch, centroid, fit.
+// One frame on one block: seed from the argmax word, patch, centroid, fit.
+// buf: side^2 floats (the box, then the window); lab: side^2 bytes (the
+// patch), the same memory as the model values zb, which come after it.
 __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long key, long long f, float *buf,
-                                          uint8_t *lab, double *ne_cur, int lane) {
+                                          uint8_t *lab, unsigned char *zb, FitShared &s) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int n = a.n;
   const float *fr = a.in + f * (long long)n * n;
   double *out = a.out + f * 8;
   auto not_found = [&]() {
-    if (lane < 8) out[lane] = 0.0;
-    if (lane == 0 && a.iters) a.iters[f] = 0;
+    if (tid < 8) out[tid] = 0.0;
+    if (tid == 0 && a.iters) a.iters[f] = 0;
   };
   if (key == KEY_NONFINITE) {
     not_found();
@@ -472,7 +575,7 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
   }
   const long long seed = (long long)(~(uint32_t)(key & 0xffffffffull));
   if (key == 0ull || seed >= (long long)n * n) {   // no maximum recorded: cannot happen for n >= 1
-    if (lane == 0) atomicOr(a.status, STATUS_INTERNAL);
+    if (tid == 0) atomicOr(a.status, STATUS_INTERNAL);
     not_found();
     return;
   }
@@ -483,77 +586,96 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
 
   // ---- patch: flood fill of the pixels above the threshold ----------------
   // lab: 0 below the threshold, 2 above and not (yet) reached, 1 in the patch
-  __syncwarp();   // the previous frame's reads of buf and lab are done
-  for (int i = lane; i < H * W; i += 32) {
+  const int si = (r0 - rlo) * W + (c0 - clo);
+  for (int i = tid; i < H * W; i += FIT_THREADS) {
     const int r = i / W, c = i - r * W;
     const float v = fr[(long long)(r + rlo) * n + (c + clo)];
     buf[i] = v;
-    lab[i] = (double)v > th ? 2 : 0;
+    lab[i] = (double)v > th ? (i == si ? 1 : 2) : 0;
   }
-  __syncwarp();
-  const int si = (r0 - rlo) * W + (c0 - clo);
+  if (tid == 0) s.touch = 0;
+  __syncthreads();
   if (lab[si] == 0) {   // the seed itself is not above the threshold
     not_found();
     return;
   }
-  __syncwarp();
-  if (lane == 0) lab[si] = 1;
-  __syncwarp();
   for (int sweep = 0; sweep <= H * W; sweep++) {
-    bool changed = false;
+    int changed = 0;
+    // 32 pixels a thread at a time: all found against the same labels, then
+    // all marked
+    for (int b = 0; b < H * W; b += 32 * FIT_THREADS) {
+      uint32_t reached = 0;
+      for (int i = b + tid, k = 0; k < 32 && i < H * W; i += FIT_THREADS, k++) {
+        if (lab[i] != 2) continue;
+        const int r = i / W, c = i - r * W;
+        bool nb = false;
+        for (int dr = -1; dr <= 1; dr++)
+          for (int dc = -1; dc <= 1; dc++) {
+            const int rr = r + dr, cc = c + dc;
+            if ((dr || dc) && rr >= 0 && rr < H && cc >= 0 && cc < W && lab[rr * W + cc] == 1) nb = true;
+          }
+        if (nb) reached |= 1u << k;
+      }
+      __syncthreads();
+      changed |= reached != 0;
+      for (; reached; reached &= reached - 1) lab[b + tid + (__ffs(reached) - 1) * FIT_THREADS] = 1;
+      __syncthreads();
+    }
+    if (!__syncthreads_or(changed)) break;
+  }
+  // the four sums, one to a warp (each in the order of 32 strided partials)
+  if (wid < 4) {
+    double acc = 0.0;
+    bool touch = false;
     for (int i = lane; i < H * W; i += 32) {
-      if (lab[i] != 2) continue;
+      if (lab[i] != 1) continue;
       const int r = i / W, c = i - r * W;
-      bool nb = false;
-      for (int dr = -1; dr <= 1; dr++)
-        for (int dc = -1; dc <= 1; dc++) {
-          const int rr = r + dr, cc = c + dc;
-          if ((dr || dc) && rr >= 0 && rr < H && cc >= 0 && cc < W && lab[rr * W + cc] == 1) nb = true;
-        }
-      if (nb) {
-        lab[i] = 1;
-        changed = true;
+      const double v = buf[i];
+      if (wid == 0) {
+        acc += 1.0;
+        touch |= (r == 0 && rlo > 0) || (r == H - 1 && rhi < n - 1) || (c == 0 && clo > 0) || (c == W - 1 && chi < n - 1);
+      } else if (wid == 1) {
+        acc += v;
+      } else {
+        acc += v * (double)(wid == 2 ? c + clo : r + rlo);
       }
     }
-    __syncwarp();
-    if (!__any_sync(0xffffffffu, changed)) break;
+    acc = warp_sum(acc);
+    if (lane == 0) s.patch[wid] = acc;
+    if (touch) s.touch = 1;
   }
-  double cnt = 0.0, sv = 0.0, sx = 0.0, sy = 0.0;
-  bool touch = false;
-  for (int i = lane; i < H * W; i += 32) {
-    if (lab[i] != 1) continue;
-    const int r = i / W, c = i - r * W;
-    const double v = buf[i];
-    cnt += 1.0;
-    sv += v;
-    sx += v * (double)(c + clo);
-    sy += v * (double)(r + rlo);
-    touch |= (r == 0 && rlo > 0) || (r == H - 1 && rhi < n - 1) || (c == 0 && clo > 0) || (c == W - 1 && chi < n - 1);
-  }
-  cnt = warp_sum(cnt);
-  sv = warp_sum(sv);
-  sx = warp_sum(sx);
-  sy = warp_sum(sy);
-  const int size = (int)cnt;
-  if (__any_sync(0xffffffffu, touch) || size < a.min_size || size > a.max_size) {
+  __syncthreads();
+  const int size = (int)s.patch[0];
+  if (s.touch || size < a.min_size || size > a.max_size) {
     not_found();
     return;
   }
-  const double cx = sx / sv, cy = sy / sv;
+  const double sv = s.patch[1];
+  const double cx = s.patch[2] / sv, cy = s.patch[3] / sv;
 
   // ---- Moffat fit ---------------------------------------------------------
-  const int rc = (int)floor(cy + 0.5), cc = (int)floor(cx + 0.5), w = a.w;
+  // (a patch with values of either sign, from a threshold below zero, can have
+  // its centroid anywhere: the window may then be empty)
+  const int far = 1 << 30, w = a.w;
+  const int rc = max(min((int)floor(cy + 0.5), far), -far), cc = max(min((int)floor(cx + 0.5), far), -far);
   const int wr0 = max(rc - w, 0), wr1 = min(rc + w, n - 1), wc0 = max(cc - w, 0), wc1 = min(cc + w, n - 1);
-  const int WH = wr1 - wr0 + 1, WW = wc1 - wc0 + 1;
-  __syncwarp();   // the box reads are done: the buffer now takes the window
-  float lmin = INFINITY;
-  for (int i = lane; i < WH * WW; i += 32) {
+  const int WH = max(wr1 - wr0 + 1, 0), WW = max(wc1 - wc0 + 1, 0);
+  // the box reads are done: the buffer now takes the window
+  for (int i = tid; i < WH * WW; i += FIT_THREADS) {
     const int r = i / WW, c = i - r * WW;
-    const float v = fr[(long long)(r + wr0) * n + (c + wc0)];
-    buf[i] = v;
-    lmin = fminf(lmin, v);
+    buf[i] = fr[(long long)(r + wr0) * n + (c + wc0)];
   }
-  __syncwarp();
+  __syncthreads();
+  if (wid > 0) {   // evaluate what warp 0 asks for
+    for (;;) {
+      fit_sync();
+      const int mode = s.mode;
+      if (mode == EVAL_DONE) return;
+      window_pass_shared(mode, s, zb, buf, WH, WW, wr0, wc0);
+    }
+  }
+  float lmin = INFINITY;
+  for (int i = lane; i < WH * WW; i += 32) lmin = fminf(lmin, buf[i]);
   const double bg = warp_min(lmin);
   double i0 = 0.0;
   for (int i = lane; i < WH * WW; i += 32) i0 += (double)buf[i] - bg;
@@ -565,10 +687,11 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
   // system well away from the FP32 noise of J^T J).  Phase B: the FP64
   // iteration of the oracle from there, which converges in a few steps to
   // the same minimum.
-  const int it_a = lm_loop<true>(p, cost, ne_cur, 1e-6, 1e-7, buf, WH, WW, wr0, wc0, lane);
-  const int it_b = lm_loop<false>(p, cost, ne_cur, 1e-12, 1e-14, buf, WH, WW, wr0, wc0, lane);
+  const int it_a = lm_loop<true>(p, cost, 1e-6, 1e-7, s, zb, buf, WH, WW, wr0, wc0);
+  const int it_b = lm_loop<false>(p, cost, 1e-12, 1e-14, s, zb, buf, WH, WW, wr0, wc0);
   const int it = it_a + it_b;
   if (lane == 0) {
+    s.mode = EVAL_DONE;
     out[0] = 1.0;
     out[1] = p[1];
     out[2] = p[2];
@@ -579,28 +702,33 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
     out[7] = p[5];
     if (a.iters) a.iters[f] = it;
   }
+  fit_sync();
 }
 
-// Persistent warps: each takes the next frame from the counter after the
-// per-frame words (no waiting on other warps).
-__global__ void __launch_bounds__(FIT_WARPS * 32) register_fit_kernel(const RegArgs a,
+// Shared memory of a block: side^2 floats, then the labels or the model values.
+__host__ __device__ inline size_t fit_buf_bytes(int side) { return ((size_t)side * side * 4 + 15) & ~(size_t)15; }
+__host__ __device__ inline size_t fit_smem_bytes(int side) {
+  const size_t lab = ((size_t)side * side + 15) & ~(size_t)15, z = (size_t)FIT_TILE * FIT_Z * sizeof(double);
+  return fit_buf_bytes(side) + (lab > z ? lab : z);
+}
+
+// Persistent blocks: each takes the next frame from the counter after the
+// per-frame words (no waiting on other blocks).
+__global__ void __launch_bounds__(FIT_THREADS, 3) register_fit_kernel(const RegArgs a,
                                                                       unsigned long long *__restrict__ keys,
                                                                       int side) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int S2 = side * side;
-  const size_t per_warp = (((size_t)S2 * 5 + 15) & ~(size_t)15) + 27 * sizeof(double);
-  unsigned char *base = smem + (size_t)wid * per_warp;
-  float *buf = reinterpret_cast<float *>(base);
-  uint8_t *lab = reinterpret_cast<uint8_t *>(buf + S2);
-  double *ne_cur = reinterpret_cast<double *>(base + (((size_t)S2 * 5 + 15) & ~(size_t)15));
+  __shared__ FitShared s;
+  float *buf = reinterpret_cast<float *>(smem);
+  unsigned char *zb = smem + fit_buf_bytes(side);
   unsigned long long *counter = keys + a.T;
   for (;;) {
-    long long f = 0;
-    if (lane == 0) f = (long long)atomicAdd(counter, 1ull);
-    f = __shfl_sync(0xffffffffu, f, 0);
+    __syncthreads();   // the frame before is done with the shared memory
+    if (threadIdx.x == 0) s.frame = (long long)atomicAdd(counter, 1ull);
+    __syncthreads();
+    const long long f = s.frame;
     if (f >= a.T) break;
-    fit_frame(a, keys[f], f, buf, lab, ne_cur, lane);
+    fit_frame(a, keys[f], f, buf, zb, zb, s);
   }
 }
 
@@ -623,20 +751,18 @@ cudaError_t launch_register_argmax(const RegArgs &a, unsigned long long *keys, c
 cudaError_t launch_register_fit(const RegArgs &a, unsigned long long *keys, cudaStream_t st) {
   if (a.T <= 0) return cudaSuccess;
   const int side = 2 * (a.R > a.w ? a.R : a.w) + 1;
-  const size_t per_warp = (((size_t)side * side * 5 + 15) & ~(size_t)15) + 27 * sizeof(double);
-  const size_t smem = per_warp * FIT_WARPS;
+  const size_t smem = fit_smem_bytes(side);
   cudaError_t e = cudaFuncSetAttribute(register_fit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev = 0, sms = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, register_fit_kernel, FIT_WARPS * 32, smem)) !=
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, register_fit_kernel, FIT_THREADS, smem)) !=
       cudaSuccess)
     return e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const long long need = (a.T + FIT_WARPS - 1) / FIT_WARPS;
   long long grid = (long long)(per_sm > 0 ? per_sm : 1) * sms;
-  if (grid > need) grid = need;
-  register_fit_kernel<<<(unsigned)grid, FIT_WARPS * 32, smem, st>>>(a, keys, side);
+  if (grid > a.T) grid = a.T;
+  register_fit_kernel<<<(unsigned)grid, FIT_THREADS, smem, st>>>(a, keys, side);
   return cudaGetLastError();
 }
 
