@@ -233,7 +233,15 @@ int end_call(graphic_ctx *c) {
   return GRAPHIC_OK;
 }
 
-constexpr size_t kCopyChunkMB = 256;   // host -> device copy pieces of graphic_reduce_host
+// Frames of one host -> device copy piece of graphic_reduce_host: an eighth of
+// the cube, so that only the last eighth's shift is left when the copy ends
+// (250 x 512 x 512: 4128 us, in one piece of 256 MiB 4427), from 16 MiB (two
+// passes over it still fill the chip) to 256 MiB (an eighth of a survey cube).
+long long copy_piece_frames(long long T, size_t bytes_per_frame) {
+  const size_t eighth = (size_t)T * bytes_per_frame / 8;
+  const size_t piece = std::min<size_t>(std::max<size_t>(eighth, (size_t)16 << 20), (size_t)256 << 20);
+  return std::max<long long>(1, std::min<long long>(T, (long long)(piece / bytes_per_frame)));
+}
 
 long long chunk_frames(const graphic_ctx *c, long long T, size_t bytes_per_frame) {
   size_t budget = (size_t)c->chunk_mb << 20;
@@ -273,27 +281,27 @@ namespace {
 // Enqueue the two shift passes for frames [0, T) with parameters at device
 // pointers p_dx, p_dy.  in -> out (out may equal in); in_fs / out_fs: the
 // frame strides in elements (0: n*n).
-int enqueue_shift(graphic_ctx *c, const float *in, float *out, int64_t T, int32_t n, const double *p_dx,
-                  const double *p_dy, long long in_fs = 0, long long out_fs = 0) {
-  const long long NN = (long long)n * n;
-  if (!in_fs) in_fs = NN;
-  if (!out_fs) out_fs = NN;
-  const long long ch = chunk_frames(c, T, (size_t)NN * sizeof(float));
-  // per-frame shift parameters of both passes, once for all frames
+// The per-frame shift parameters of both passes for T frames, the x table
+// then the y table, to c->d_lparam.
+int shift_params(graphic_ctx *c, int64_t T, int32_t n, const double *p_dx, const double *p_dy) {
   const size_t pb = line_params_bytes(SHIFT_X, n, T);
   int rc = ensure(c, (void **)&c->d_lparam, &c->lparam_bytes, 2 * pb, false);
   if (rc) return rc;
-  {
-    LineArgs a{};
-    a.p0 = p_dx;
-    a.p1 = p_dy;
-    a.n = n;
-    cudaError_t e = launch_line_params(SHIFT_X, a, T, c->d_lparam, c->stream);
-    if (e == cudaSuccess) e = launch_line_params(SHIFT_Y, a, T, c->d_lparam + pb, c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "shift parameters");
-  }
-  for (long long f0 = 0; f0 < T; f0 += ch) {
-    const long long nf = std::min<long long>(ch, T - f0);
+  LineArgs a{};
+  a.p0 = p_dx;
+  a.p1 = p_dy;
+  a.n = n;
+  cudaError_t e = launch_line_params(STEP_SHIFT, a, T, c->d_lparam, c->d_lparam + pb, c->stream);
+  return e == cudaSuccess ? GRAPHIC_OK : cuda_fail(e, "shift parameters");
+}
+
+// Both passes of frames [f0, f1) of the T that shift_params was called for.
+int shift_passes(graphic_ctx *c, const float *in, float *out, int64_t T, int64_t f0, int64_t f1, int32_t n,
+                 const double *p_dx, const double *p_dy, long long in_fs, long long out_fs) {
+  const size_t pb = line_params_bytes(SHIFT_X, n, T);
+  const long long ch = chunk_frames(c, T, (size_t)n * n * sizeof(float));
+  for (; f0 < f1; f0 += ch) {
+    const long long nf = std::min<long long>(ch, f1 - f0);
     LineArgs a{};
     a.in = in + f0 * in_fs;
     a.out = out + f0 * out_fs;
@@ -318,6 +326,14 @@ int enqueue_shift(graphic_ctx *c, const float *in, float *out, int64_t T, int32_
     if (e != cudaSuccess) return cuda_fail(e, "shift y pass");
   }
   return GRAPHIC_OK;
+}
+
+int enqueue_shift(graphic_ctx *c, const float *in, float *out, int64_t T, int32_t n, const double *p_dx,
+                  const double *p_dy, long long in_fs = 0, long long out_fs = 0) {
+  const long long NN = (long long)n * n;
+  int rc = shift_params(c, T, n, p_dx, p_dy);
+  if (rc) return rc;
+  return shift_passes(c, in, out, T, 0, T, n, p_dx, p_dy, in_fs ? in_fs : NN, out_fs ? out_fs : NN);
 }
 
 // --- rotate -----------------------------------------------------------------
@@ -369,8 +385,7 @@ int enqueue_rotate(graphic_ctx *c, const float *in, float *out, int64_t T, int32
     a.status = c->d_status;
     a.n = n;
     {
-      cudaError_t e = launch_line_params(ROT_P1, a, nf, c->d_lparam, c->stream);
-      if (e == cudaSuccess) e = launch_line_params(ROT_P2, a, nf, c->d_lparam + pb13, c->stream);
+      cudaError_t e = launch_line_params(STEP_ROTATE, a, nf, c->d_lparam, c->d_lparam + pb13, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "shear parameters");
     }
     a.lp_tab = c->d_lparam;
@@ -695,19 +710,19 @@ int reduce_device(graphic_ctx *c, const float *in, float *work, int64_t T, int32
     // the copies start after everything already on the compute stream
     CK(cudaEventRecord(c->ev_copy, c->stream));
     CK(cudaStreamWaitEvent(c->s_copy, c->ev_copy, 0));
-    // copies in pieces of kCopyChunkMB, each piece's shift launched as soon as
-    // it lands (the copy, not the shift, bounds this path)
+    // copies in pieces, each piece's shift launched as soon as it lands (the
+    // copy, not the shift, bounds this path)
+    if ((rc = shift_params(c, T, n, at<double>(c, o_dx), at<double>(c, o_dy)))) return rc;
     const size_t NN = (size_t)n * n;
-    const long long ch = std::max<long long>(1, std::min<long long>(T, (long long)((kCopyChunkMB << 20) /
-                                                                                    (NN * sizeof(float)))));
+    const long long ch = copy_piece_frames(T, NN * sizeof(float));
     for (long long f0 = 0; f0 < T; f0 += ch) {
       const long long nf = std::min<long long>(ch, T - f0);
       CK(cudaMemcpyAsync(const_cast<float *>(in) + f0 * NN, host_in + f0 * NN, nf * NN * sizeof(float),
                          cudaMemcpyHostToDevice, c->s_copy));
       CK(cudaEventRecord(c->ev_copy, c->s_copy));
       CK(cudaStreamWaitEvent(c->stream, c->ev_copy, 0));
-      if ((rc = enqueue_shift(c, in + f0 * NN, work + f0 * NN, nf, n, at<double>(c, o_dx) + f0,
-                              at<double>(c, o_dy) + f0)))
+      if ((rc = shift_passes(c, in, work, T, f0, f0 + nf, n, at<double>(c, o_dx), at<double>(c, o_dy), (long long)NN,
+                             (long long)NN)))
         return rc;
     }
   }
@@ -1094,8 +1109,7 @@ int batch_grouped(graphic_ctx *c, const graphic_batch_item *items, int32_t n_ite
         a.p0 = at<double>(c, o_dx) + w.f0;
         a.p1 = at<double>(c, o_dy) + w.f0;
         const size_t pb1 = line_params_bytes(SHIFT_X, w.n, w.nf);
-        e = launch_line_params(SHIFT_X, a, w.nf, tab, st);
-        if (e == cudaSuccess) e = launch_line_params(SHIFT_Y, a, w.nf, tab + pb1, st);
+        e = launch_line_params(STEP_SHIFT, a, w.nf, tab, tab + pb1, st);
         a.lp_lines = 1;
         a.lp_tab = tab;
         if (e == cudaSuccess) e = line_pass(c, SHIFT_X, a, w.nf, st);
@@ -1116,8 +1130,7 @@ int batch_grouped(graphic_ctx *c, const graphic_batch_item *items, int32_t n_ite
         b.out = slot;
         b.out_fstride = NM;
         const size_t pb13 = line_params_bytes(ROT_P1, w.n, w.nf);
-        e = launch_line_params(ROT_P1, b, w.nf, tab, st);
-        if (e == cudaSuccess) e = launch_line_params(ROT_P2, b, w.nf, tab + pb13, st);
+        e = launch_line_params(STEP_ROTATE, b, w.nf, tab, tab + pb13, st);
         b.lp_tab = tab;
         b.lp_lines = line_params_lines(ROT_P1, w.n);
         if (e == cudaSuccess) e = line_pass(c, ROT_P1, b, w.nf, st);

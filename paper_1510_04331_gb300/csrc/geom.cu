@@ -1276,15 +1276,20 @@ bool configure_m() {
 }  // namespace
 
 // One thread per line: the line's shift parameters in FP64 (the arithmetic
-// each CTA of the passes would otherwise do on GB300's narrow FP64 pipe).
-template <int KIND>
-__global__ void __launch_bounds__(256) line_param_kernel(const LineArgs a, long long n_frames, int lines,
-                                                        LineParam *out) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_frames * lines) return;
-  const long long f = idx / lines;
-  const int line = (int)(idx - f * lines);
-  make_param(out[idx], line_shift<KIND>(a, f, line, a.n), 2 * a.n);
+// each CTA of the passes would otherwise do on GB300's narrow FP64 pipe).  Both
+// tables of a step in one launch: the lines of kind K1, then those of K2
+// (a launch each: 59 us against 56 for the shift of one 512 x 512 frame).
+template <int K1, int K2>
+__global__ void __launch_bounds__(256) line_param_kernel(const LineArgs a, long long n_frames, int lines1, int lines2,
+                                                        LineParam *out1, LineParam *out2) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x, n1 = n_frames * lines1;
+  if (idx < n1) {
+    const long long f = idx / lines1;
+    make_param(out1[idx], line_shift<K1>(a, f, (int)(idx - f * lines1), a.n), 2 * a.n);
+  } else if (idx - n1 < n_frames * lines2) {
+    const long long i2 = idx - n1, f = i2 / lines2;
+    make_param(out2[i2], line_shift<K2>(a, f, (int)(i2 - f * lines2), a.n), 2 * a.n);
+  }
 }
 
 int line_params_lines(LineKind kind, int n) {
@@ -1295,19 +1300,18 @@ size_t line_params_bytes(LineKind kind, int n, long long n_frames) {
   return (size_t)n_frames * line_params_lines(kind, n) * sizeof(LineParam);
 }
 
-cudaError_t launch_line_params(LineKind kind, const LineArgs &a, long long n_frames, void *out, cudaStream_t st) {
-  const int lines = line_params_lines(kind, a.n);
-  const long long total = n_frames * lines;
+cudaError_t launch_line_params(LineStep step, const LineArgs &a, long long n_frames, void *out1, void *out2,
+                               cudaStream_t st) {
+  const LineKind k1 = step == STEP_SHIFT ? SHIFT_X : ROT_P1, k2 = step == STEP_SHIFT ? SHIFT_Y : ROT_P2;
+  const int l1 = line_params_lines(k1, a.n), l2 = line_params_lines(k2, a.n);
+  const long long total = n_frames * (l1 + l2);
   if (total == 0) return cudaSuccess;
   const unsigned grid = (unsigned)((total + 255) / 256);
-  LineParam *o = reinterpret_cast<LineParam *>(out);
-  switch (kind) {
-    case SHIFT_X: line_param_kernel<SHIFT_X><<<grid, 256, 0, st>>>(a, n_frames, lines, o); break;
-    case SHIFT_Y: line_param_kernel<SHIFT_Y><<<grid, 256, 0, st>>>(a, n_frames, lines, o); break;
-    case ROT_P1:
-    case ROT_P3: line_param_kernel<ROT_P1><<<grid, 256, 0, st>>>(a, n_frames, lines, o); break;
-    case ROT_P2: line_param_kernel<ROT_P2><<<grid, 256, 0, st>>>(a, n_frames, lines, o); break;
-  }
+  LineParam *o1 = reinterpret_cast<LineParam *>(out1), *o2 = reinterpret_cast<LineParam *>(out2);
+  if (step == STEP_SHIFT)
+    line_param_kernel<SHIFT_X, SHIFT_Y><<<grid, 256, 0, st>>>(a, n_frames, l1, l2, o1, o2);
+  else
+    line_param_kernel<ROT_P1, ROT_P2><<<grid, 256, 0, st>>>(a, n_frames, l1, l2, o1, o2);
   return cudaGetLastError();
 }
 

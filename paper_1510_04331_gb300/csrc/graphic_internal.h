@@ -115,12 +115,15 @@ int geom_init_device();   // uploads the twiddle tables of the current device (0
 cudaError_t launch_line_pass(LineKind kind, const LineArgs &a, long long n_frames, cudaStream_t st,
                              int variant_1024 = 1);
 // Parameter tables for the line passes (geom.cu): the parameters of every
-// line of n_frames frames of pass `kind` (ROT_P1 and ROT_P3 share theirs),
-// computed in FP64 by one thread per line into `out`, line_params_bytes(kind,
-// n, n_frames) bytes; the lines per frame of the table is line_params_lines.
+// line of n_frames frames of both kinds of pass of a step (out1: SHIFT_X or
+// ROT_P1, which ROT_P3 shares; out2: SHIFT_Y or ROT_P2), computed in FP64 by
+// one thread per line, line_params_bytes(kind, n, n_frames) bytes each; the
+// lines per frame of a table is line_params_lines.
 int line_params_lines(LineKind kind, int n);
 size_t line_params_bytes(LineKind kind, int n, long long n_frames);
-cudaError_t launch_line_params(LineKind kind, const LineArgs &a, long long n_frames, void *out, cudaStream_t st);
+enum LineStep { STEP_SHIFT, STEP_ROTATE };
+cudaError_t launch_line_params(LineStep step, const LineArgs &a, long long n_frames, void *out1, void *out2,
+                               cudaStream_t st);
 
 // Uneven batches (one persistent launch): per-frame descriptor ...
 struct BatchFrame {

@@ -290,8 +290,8 @@ int start_copy_in(graphic_server *s, Req *r) {
   a.n = r->n;
   a.status = s->d_status + r->slot;
   const size_t pb = graphic::line_params_bytes(graphic::SHIFT_X, r->n, T);
-  if (e == cudaSuccess) e = graphic::launch_line_params(graphic::SHIFT_X, a, T, plan + r->o_ptab, s->s_in);
-  if (e == cudaSuccess) e = graphic::launch_line_params(graphic::SHIFT_Y, a, T, plan + r->o_ptab + pb, s->s_in);
+  if (e == cudaSuccess)
+    e = graphic::launch_line_params(graphic::STEP_SHIFT, a, T, plan + r->o_ptab, plan + r->o_ptab + pb, s->s_in);
   const int64_t NN = (int64_t)r->n * r->n;
   const int64_t ch = std::max<int64_t>(1, std::min<int64_t>(T, ((int64_t)256 << 20) / (NN * (int64_t)sizeof(float))));
   for (int64_t f0 = 0; f0 < T && e == cudaSuccess; f0 += ch) {
