@@ -280,6 +280,10 @@ cudaError_t launch_register_fit(const RegArgs &a, unsigned long long *keys, cuda
 // out: ceil(T / B) frames; *launched receives the kernel count
 cudaError_t launch_bin_median(const float *in, float *out, long long T, int n, int B, int *status, cudaStream_t st,
                               int *launched = nullptr);
+// Medians of groups of B <= 64 frames, fs elements between frames (even, and
+// in and out 8-byte aligned: pixels are taken in pairs).
+cudaError_t launch_median_network(const float *in, float *out, long long T, int n, long long fs, int B, int *status,
+                                  cudaStream_t st);
 // pos: [T][n_comp] (x, y) FP64; win: [T][n_comp] (row, col) of the window
 // centre; amp: [T][n_comp] Moffat peak; shape: [T] (1 / alpha^2, beta), FP32
 cudaError_t launch_inject(float *cube, long long T, int n, int n_comp, const double *pos, const int *win,

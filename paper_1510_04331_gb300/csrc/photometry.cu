@@ -13,7 +13,8 @@
 //    branch of its own for full bins, is what brings it there: with the
 //    slot tests between the loads it ran at 4.7 TB/s.
 //    Groups of more than 64 frames go to the median collapse kernel, one
-//    launch per group.
+//    launch per group; the collapse of at most 64 frames comes here as one
+//    group.
 //  * inject_kernel: one block per frame; companions in turn (a barrier
 //    between them, so overlapping windows never race), each over its window
 //    of (2 half + 1)^2 pixels; positions and windows come from the FP64 host
@@ -39,23 +40,23 @@ constexpr int BIN_THREADS = 128;
 // above).  All loads are issued before the first comparison.
 template <int W, int V>
 __global__ void __launch_bounds__(BIN_THREADS) bin_median_kernel(const float *__restrict__ in, float *__restrict__ out,
-                                                                 long long T, long long nn, int B,
+                                                                 long long T, long long nn, long long fs, int B,
                                                                  unsigned blocks_per_group, int *status) {
   const long long g = blockIdx.x / blocks_per_group;
   const long long p = ((long long)(blockIdx.x % blocks_per_group) * BIN_THREADS + threadIdx.x) * V;
   if (p >= nn) return;
   const long long f0 = g * B;
   const int m = (int)((T - f0) < B ? (T - f0) : B);
-  const float *src = in + f0 * nn + p;
+  const float *src = in + f0 * fs + p;
   float v[V][W];
   float acc = 0.f;   // 0 while every value is finite: v * 0 is NaN for NaN and infinities
   auto load = [&](int i) {
     if constexpr (V == 2) {
-      const float2 x = __ldcs(reinterpret_cast<const float2 *>(src + (long long)i * nn));
+      const float2 x = __ldcs(reinterpret_cast<const float2 *>(src + (long long)i * fs));
       v[0][i] = x.x;
       v[V - 1][i] = x.y;
     } else {
-      v[0][i] = __ldcs(src + (long long)i * nn);
+      v[0][i] = __ldcs(src + (long long)i * fs);
     }
   };
   if (m == W) {   // a full bin of the network's own width: no slot to test
@@ -146,17 +147,41 @@ __global__ void aperture_kernel(const float *__restrict__ img, int n, const doub
 }
 
 template <int W, int V>
-cudaError_t bin_launch(const float *in, float *out, long long T, long long nn, int B, int *status,
+cudaError_t bin_launch(const float *in, float *out, long long T, long long nn, long long fs, int B, int *status,
                        cudaStream_t st) {
   const long long G = (T + B - 1) / B;
   const long long bpg = (nn + BIN_THREADS * V - 1) / (BIN_THREADS * V);
   // one block per (bin, 128 or 256 pixels); the limit of the one-pixel form holds for both
   if (G * ((nn + BIN_THREADS - 1) / BIN_THREADS) > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  bin_median_kernel<W, V><<<(unsigned)(G * bpg), BIN_THREADS, 0, st>>>(in, out, T, nn, B, (unsigned)bpg, status);
+  bin_median_kernel<W, V><<<(unsigned)(G * bpg), BIN_THREADS, 0, st>>>(in, out, T, nn, fs, B, (unsigned)bpg, status);
   return cudaGetLastError();
 }
 
 }  // namespace
+
+// Medians of groups of B <= 64 frames, fs elements apart.
+cudaError_t launch_median_network(const float *in, float *out, long long T, int n, long long fs, int B, int *status,
+                                  cudaStream_t st) {
+  const long long nn = (long long)n * n;
+  // the narrowest network that holds a bin (the comparators grow faster than
+  // W); two pixels per thread (8-byte loads) up to 32 values: 1000 frames of
+  // 512 x 512 in 165 us against 195 for B = 10, 185 / 194 for 32; from 40 on
+  // their registers cost more (B = 50: 240 us with one pixel, 260 with two)
+  if (B <= 2) return bin_launch<2, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 4) return bin_launch<4, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 6) return bin_launch<6, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 8) return bin_launch<8, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 10) return bin_launch<10, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 12) return bin_launch<12, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 16) return bin_launch<16, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 20) return bin_launch<20, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 24) return bin_launch<24, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 32) return bin_launch<32, 2>(in, out, T, nn, fs, B, status, st);
+  if (B <= 40) return bin_launch<40, 1>(in, out, T, nn, fs, B, status, st);
+  if (B <= 50) return bin_launch<50, 1>(in, out, T, nn, fs, B, status, st);
+  if (B <= 64) return bin_launch<64, 1>(in, out, T, nn, fs, B, status, st);
+  return cudaErrorInvalidValue;
+}
 
 cudaError_t launch_bin_median(const float *in, float *out, long long T, int n, int B, int *status, cudaStream_t st,
                               int *launched) {
@@ -165,23 +190,7 @@ cudaError_t launch_bin_median(const float *in, float *out, long long T, int n, i
   const long long nn = (long long)n * n;
   const long long G = (T + B - 1) / B;
   cudaError_t e;
-  // the narrowest network that holds a bin (the comparators grow faster than
-  // W); two pixels per thread (8-byte loads) up to 32 values: 1000 frames of
-  // 512 x 512 in 165 us against 195 for B = 10, 185 / 194 for 32; from 40 on
-  // their registers cost more (B = 50: 240 us with one pixel, 260 with two)
-  if (B <= 2) e = bin_launch<2, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 4) e = bin_launch<4, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 6) e = bin_launch<6, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 8) e = bin_launch<8, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 10) e = bin_launch<10, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 12) e = bin_launch<12, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 16) e = bin_launch<16, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 20) e = bin_launch<20, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 24) e = bin_launch<24, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 32) e = bin_launch<32, 2>(in, out, T, nn, B, status, st);
-  else if (B <= 40) e = bin_launch<40, 1>(in, out, T, nn, B, status, st);
-  else if (B <= 50) e = bin_launch<50, 1>(in, out, T, nn, B, status, st);
-  else if (B <= 64) e = bin_launch<64, 1>(in, out, T, nn, B, status, st);
+  if (B <= 64) e = launch_median_network(in, out, T, n, nn, B, status, st);
   else {
     for (long long g = 0; g < G; g++) {
       CollapseArgs a{};

@@ -1,7 +1,8 @@
 // select_common.cuh -- device helpers shared by the selection kernels (the
 // median collapse and master sky of median.cu, the median PSF of psf_band.cu
-// and psf_general.cu, the binning of photometry.cu): IEEE total-order keys, asynchronous shared-memory copies, bit
-// selection.  Each translation unit gets its own copy (anonymous namespace).
+// and psf_general.cu, the binning of photometry.cu): IEEE total-order keys,
+// asynchronous shared-memory copies, median networks, bit selection.  Each
+// translation unit gets its own copy (anonymous namespace).
 #pragma once
 
 #include <cuda_runtime.h>
