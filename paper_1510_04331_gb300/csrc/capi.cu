@@ -482,7 +482,12 @@ int graphic::plan_adi(const double *parang, int64_t T, double fwhm, double n_fwh
   for (int64_t t = 0; t < T; t++) ap.perm[t] = (int)t;
   std::stable_sort(ap.perm.begin(), ap.perm.end(), [&](int x, int y) { return parang[x] < parang[y]; });
   ap.edge2.resize(n_edges);
-  for (int i = 0; i < n_edges; i++) ap.edge2[i] = edges[i] * edges[i];
+  ap.iedge2.resize(n_edges);
+  for (int i = 0; i < n_edges; i++) {
+    ap.edge2[i] = edges[i] * edges[i];
+    const double up = ceil(ap.edge2[i]);
+    ap.iedge2[i] = up < (double)INT32_MAX ? (int)up : INT32_MAX;
+  }
   // time windows [A, B) in the angle order (the whole order without a time gate)
   ap.ab.clear();
   std::vector<int> wa(T, 0), wb(T, (int)T);
@@ -594,7 +599,7 @@ struct AdiOffsets {
 
 AdiOffsets add_adi_plan(PlanBuilder &pb, const AdiPlanHost &ap, int64_t T) {
   AdiOffsets o{};
-  o.e2 = pb.add(ap.edge2.data(), ap.edge2.size() * sizeof(double));
+  o.e2 = pb.add(ap.iedge2.data(), ap.iedge2.size() * sizeof(int));
   o.perm = pb.add(ap.perm.data(), T * sizeof(int));
   o.lr = pb.add(ap.lr.data(), ap.lr.size() * sizeof(int));
   o.band = pb.add(ap.band.data(), ap.band.size() * sizeof(int));
@@ -654,7 +659,7 @@ int enqueue_adi(graphic_ctx *c, const float *in, float *out, int64_t T, int32_t 
   a.perm = at<int>(c, o.perm);
   a.lr = at<int>(c, o.lr);
   a.ab = ap.ab.empty() ? nullptr : at<int>(c, o.ab);
-  a.edge2 = at<double>(c, o.e2);
+  a.iedge2 = at<int>(c, o.e2);
   a.band = at<int>(c, o.band);
   a.status = c->d_status;
   a.T = (int)T;

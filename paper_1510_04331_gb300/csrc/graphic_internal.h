@@ -60,6 +60,8 @@ struct AdiPlanHost {
   std::vector<int> lr;       // [A][T][2]
   std::vector<int> ab;       // [T][2] time windows (empty without a time gate)
   std::vector<double> edge2; // [A+1]
+  std::vector<int> iedge2;   // [A+1] the same rounded up: squared radii of pixels are whole numbers, so
+                             // edge2 <= rho2 and iedge2 <= rho2 are the same (INT_MAX beyond the range)
   std::vector<int> band;     // [A][4]
   int wmax = 0;
   // band path (plan_band_path): event queries [A][T] (a_s | b_s << 16: frame s
@@ -180,7 +182,7 @@ struct AdiArgs {
   const int *lr;         // [A][T][2] (L, R) of the reference set of sorted frame s in annulus a
   const int *ab;         // [T][2] time window (A, B) of sorted frame s, A <= L <= R <= B (null: [0, T));
                          // the reference set is [A, L) u [R, B)
-  const double *edge2;   // [A+1] squared annulus edges (FP64)
+  const int *iedge2;     // [A+1] squared annulus edges, rounded up
   const int *band;       // [A][4] (blo, bhi, W, 0): full-rank band holding every median the
                          // annulus needs, W = bitmap words per lane (0: general path)
   int *status;

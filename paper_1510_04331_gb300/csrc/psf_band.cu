@@ -92,14 +92,6 @@ struct BandArgs {
   int nwt;               // ceil(T / 32)
 };
 
-__device__ __forceinline__ int annulus_of(long long p, int n, const double *edge2, int n_ann) {
-  const long long x = (p % n) - n / 2, y = (p / n) - n / 2;
-  const double rho2 = (double)(x * x + y * y);
-  for (int a = 0; a < n_ann; a++)
-    if (edge2[a] <= rho2 && rho2 < edge2[a + 1]) return a;
-  return -1;
-}
-
 // Bin of a key in a histogram linear in value from v0 with `scale` bins per
 // unit: monotone non-decreasing in the key (every step is a monotone
 // rounding), clamped to [0, 255].  A scale of 0 (empty or overflowing
@@ -188,7 +180,7 @@ __global__ void __launch_bounds__(32 * PPC, 4) band_prep_kernel(const BandArgs B
   uint32_t *below = reinterpret_cast<uint32_t *>(wb + al16(2048 + (size_t)B.cap * 8));
   __shared__ int ann_s[PPC];
 
-  if (lane == 0) ann_s[w] = annulus_of(p0 + w, a.n, a.edge2, a.n_ann);
+  if (lane == 0) ann_s[w] = annulus_of(p0 + w, a.n, a.iedge2, a.n_ann);
   // the group's 4 pixels of every frame, angle order: one 16-byte copy each,
   // in four quarters, so that the key conversion of a quarter overlaps the
   // copies of the later ones

@@ -69,20 +69,12 @@ struct GeneralArgs {
   int C;                 // queries per chunk (psf_sweep_kernel)
 };
 
-__device__ __forceinline__ int annulus_of(long long p, int n, const double *edge2, int n_ann) {
-  const long long x = (p % n) - n / 2, y = (p / n) - n / 2;
-  const double rho2 = (double)(x * x + y * y);
-  for (int a = 0; a < n_ann; a++)
-    if (edge2[a] <= rho2 && rho2 < edge2[a + 1]) return a;
-  return -1;
-}
-
 // Annuli of a segment's 8 pixels and which of its two 4-pixel groups are the
 // general path's: those with a pixel of an annulus without a band.
 __device__ __forceinline__ bool group_general(const AdiArgs &a, long long p) {
   bool g = a.wmax == 0;   // no band path at all
   for (int q = 0; q < 4 && !g; q++) {
-    const int an = annulus_of((p & ~3ll) + q, a.n, a.edge2, a.n_ann);
+    const int an = annulus_of((p & ~3ll) + q, a.n, a.iedge2, a.n_ann);
     g = an >= 0 && __ldg(&a.band[4 * an + 2]) == 0;
   }
   return g;
@@ -128,7 +120,7 @@ __global__ void __launch_bounds__(RANK_THREADS) full_rank_kernel(const GeneralAr
   if (seg < 0) return;
   const long long p0 = (long long)seg * SEG;
   if (tid < SEG)
-    ann_s[tid] = group_general(a, p0 + tid) ? annulus_of(p0 + tid, a.n, a.edge2, a.n_ann) : -1;
+    ann_s[tid] = group_general(a, p0 + tid) ? annulus_of(p0 + tid, a.n, a.iedge2, a.n_ann) : -1;
   __syncthreads();
   const size_t pb = full_pixel_bytes<BINS>(T);
   auto kA_of = [&](int q) { return reinterpret_cast<uint32_t *>(fsm + q * pb); };
@@ -376,7 +368,7 @@ __global__ void __launch_bounds__(512, 2) psf_sweep_kernel(const GeneralArgs g) 
   };
   const long long p = (long long)segment(lane / SEG) * SEG + (lane & (SEG - 1));
   const bool mine = (lane < SEG || __ldg(&u[lane / SEG]) >= 0) &&
-                    annulus_of(p, a.n, a.edge2, a.n_ann) == ann && group_general(a, p);
+                    annulus_of(p, a.n, a.iedge2, a.n_ann) == ann && group_general(a, p);
 
   auto code = [&](int s) { return (int)__ldg(&codes[s * UNIT]); };   // a signed load
   const int2 *LR = reinterpret_cast<const int2 *>(a.lr + (size_t)ann * T * 2);
@@ -553,7 +545,7 @@ __global__ void __launch_bounds__(512, 2) psf_sweep_kernel(const GeneralArgs g) 
 // every frame.  One CTA per listed segment.
 __global__ void __launch_bounds__(128) general_zero_kernel(const AdiArgs a) {
   const long long p = (long long)__ldg(&a.zero[blockIdx.x]) * SEG + (threadIdx.x & (SEG - 1));
-  if (annulus_of(p, a.n, a.edge2, a.n_ann) >= 0 || !group_general(a, p)) return;
+  if (annulus_of(p, a.n, a.iedge2, a.n_ann) >= 0 || !group_general(a, p)) return;
   for (int t = threadIdx.x / SEG; t < a.T; t += 128 / SEG) a.out[(long long)t * a.out_fs + p] = 0.f;
 }
 

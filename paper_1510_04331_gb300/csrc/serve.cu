@@ -270,7 +270,7 @@ int start_copy_in(graphic_server *s, Req *r) {
   const int64_t T = r->T;
   memcpy(hp + r->o_perm, r->ap.perm.data(), T * sizeof(int));
   memcpy(hp + r->o_lr, r->ap.lr.data(), r->ap.lr.size() * sizeof(int));
-  memcpy(hp + r->o_e2, r->ap.edge2.data(), r->ap.edge2.size() * sizeof(double));
+  memcpy(hp + r->o_e2, r->ap.iedge2.data(), r->ap.iedge2.size() * sizeof(int));
   memcpy(hp + r->o_band, r->ap.band.data(), r->ap.band.size() * sizeof(int));
   memcpy(hp + r->o_evq, r->ap.evq.data(), r->ap.evq.size() * sizeof(uint32_t));
   memcpy(hp + r->o_groups, r->ap.groups.data(), r->ap.groups.size() * sizeof(int));
@@ -442,7 +442,7 @@ void issue_iteration(graphic_server *s) {
     a.out = cube;
     a.perm = reinterpret_cast<const int *>(plan + r->o_perm);
     a.lr = reinterpret_cast<const int *>(plan + r->o_lr);
-    a.edge2 = reinterpret_cast<const double *>(plan + r->o_e2);
+    a.iedge2 = reinterpret_cast<const int *>(plan + r->o_e2);
     a.band = reinterpret_cast<const int *>(plan + r->o_band);
     a.units = reinterpret_cast<const int *>(plan + r->o_units);
     a.zero = reinterpret_cast<const int *>(plan + r->o_zero);
@@ -627,7 +627,7 @@ int graphic_server_submit(graphic_server *s, const graphic_request *rq, int64_t 
   r->o_lr = o;
   o = align16(o + r->ap.lr.size() * sizeof(int));
   r->o_e2 = o;
-  o = align16(o + r->ap.edge2.size() * sizeof(double));
+  o = align16(o + r->ap.iedge2.size() * sizeof(int));
   r->o_band = o;
   o = align16(o + r->ap.band.size() * sizeof(int));
   r->o_evq = o;
