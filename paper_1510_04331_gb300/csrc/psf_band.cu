@@ -126,20 +126,16 @@ __device__ __forceinline__ void hist_locate2(const uint32_t *hist, uint32_t r0, 
   for (int q = 0; q < 2; q++) {
     const unsigned ball = __ballot_sync(FULL, inc > rr[q]);
     const int L = ball ? __ffs(ball) - 1 : 31;
-    int bb = 0;
-    uint32_t bel = 0;
-    if (lane == L) {
-      uint32_t acc = exc;
-      bool done = false;
+    // every lane counts its bins that end at or below the rank; lane L's
+    // count is the bin
+    int bb = lane * 8;
+    uint32_t end = exc, bel = exc;
 #pragma unroll
-      for (int b = 0; b < 8; b++) {
-        if (!done && acc + h[b] > rr[q]) {
-          bb = lane * 8 + b;
-          bel = acc;
-          done = true;
-        }
-        acc += h[b];
-      }
+    for (int b = 0; b < 7; b++) {
+      end += h[b];
+      const bool past = end <= rr[q];
+      bb += past ? 1 : 0;
+      bel = past ? end : bel;
     }
     rb[q] = __shfl_sync(FULL, bb, L);
     rbel[q] = __shfl_sync(FULL, bel, L);
@@ -164,7 +160,12 @@ __host__ __device__ inline size_t prep_smem_bytes(int T, int cap, int nwt) {
   return al16((size_t)T * KS * 4) + PPC * prep_warp_bytes(cap, nwt);
 }
 
-__global__ void __launch_bounds__(32 * PPC, 4) band_prep_kernel(const BandArgs B) {
+// Registers for seven CTAs per SM (64 instead of 80, which left six): short
+// cubes, whose shared memory would allow more, wait on the chain of small
+// steps per pixel (32 frames of 512 x 512: 326 -> 273 us, 301 of 256 x 256: 201
+// -> 180, 600 of 512 x 512: 907 -> 823; nine CTAs 259, 178, 811, but 2000 frames,
+// three or four CTAs by shared memory, 3094 -> 3130).
+__global__ void __launch_bounds__(32 * PPC, 7) band_prep_kernel(const BandArgs B) {
   extern __shared__ __align__(16) unsigned char psm[];
   const AdiArgs &a = B.a;
   const int T = a.T;
