@@ -8,7 +8,8 @@
 // bit-reproducible.  Per pixel, a value-linear histogram over a sampled range
 // locates the two middle ranks, read off a short candidate list
 // (collapse2_kernel); radix selects (8-bit digits) are its exact fallback and
-// the masked (master sky) and long-cube form (collapse_kernel).
+// the masked (master sky) and long-cube form (collapse_kernel).  Up to 64
+// frames both take register networks (launch_median_network, sky_net_kernel).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
