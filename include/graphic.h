@@ -205,7 +205,8 @@ int graphic_reduce_host(graphic_ctx *ctx, const float *host_in, int64_t n_frames
  * cudaMalloc (an allocator policy that forbids it, a host application that
  * hands over only a stream and pre-allocated buffers, a path that must not
  * trigger allocator work).  Same arithmetic and result as graphic_rotate;
- * in, out: device cubes of the caller, n_frames x n x n floats; theta_deg:
+ * in, out: device cubes of the caller, n_frames x n x n floats, at any float
+ * address (16-byte aligned input is read in wider loads); theta_deg:
  * host array of n_frames doubles; stream: cudaStream_t (NULL = legacy
  * default stream); runs on the CURRENT CUDA device and waits for `stream`.
  * No context is needed.  Its working memory is a 16 MiB static device

@@ -30,6 +30,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "graphic_internal.h"
 #include "line_common.cuh"
 
@@ -407,7 +409,8 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
         } else if constexpr (KIND == SHIFT_Y) {
           z = ldf2<CG>(fin + (size_t)pos * N + line0);
         } else if constexpr (KIND == ROT_P1) {
-          z = load_rot90_pair<CG>(fin, N, q, line0, pos);
+          z = aligned(fin, 8) ? load_rot90_pair<CG>(fin, N, q, line0, pos)
+                              : load_rot90_pair<CG, false>(fin, N, q, line0, pos);
         }
       }
       if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
@@ -439,9 +442,8 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
   }
   if constexpr (KIND == ROT_P1 && STAGE) {
     // an odd number of quarter turns: the rows of rot90^q(frame) are columns
-    // of the frame.  (16-byte loads: the allocation-free rotation takes
-    // frames at any float address.)
-    staged = (q & 1) && ((uintptr_t)fin & 15) == 0;
+    // of the frame
+    staged = (q & 1) && aligned(fin, 16);
     if (staged) {
       if (q == 1) {   // element pos >= 1 of line i is frame[n - pos][i]; element 0 is zero
         stage_columns<N, LPC, TH, LBUF, CG>(fin + col0, N, stage, [](int row) { return row ? N - row : -1; });
@@ -486,26 +488,30 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
       if (bad) atomicOr(a.status, STATUS_NONFINITE);
     }
   } else {
+    auto load = [&](auto pair) {
 #pragma unroll
-    for (int m = 0; m < 16; m++) {
-      const int pos = j + m * (M / 16);
-      float2 z = make_float2(0.f, 0.f);
-      if (m * (M / 16) < NIN) {   // compile-time pruning of the zero half
-        if constexpr (KIND == SHIFT_X) {
-          z = make_float2(ldf<CG>(fin + (size_t)line0 * N + pos), ldf<CG>(fin + (size_t)(line0 + 1) * N + pos));
-        } else if constexpr (KIND == SHIFT_Y) {
-          z = ldf2<CG>(fin + (size_t)pos * N + line0);
-        } else if constexpr (KIND == ROT_P1) {
-          z = load_rot90_pair<CG>(fin, N, q, line0, pos);
-        } else if constexpr (KIND == ROT_P2) {
-          z = ldf2<CG>(fin + (size_t)pos * M + line0);
-        } else {
-          z = make_float2(ldf<CG>(fin + (size_t)line0 * M + pos), ldf<CG>(fin + (size_t)(line0 + 1) * M + pos));
+      for (int m = 0; m < 16; m++) {
+        const int pos = j + m * (M / 16);
+        float2 z = make_float2(0.f, 0.f);
+        if (m * (M / 16) < NIN) {   // compile-time pruning of the zero half
+          if constexpr (KIND == SHIFT_X) {
+            z = make_float2(ldf<CG>(fin + (size_t)line0 * N + pos), ldf<CG>(fin + (size_t)(line0 + 1) * N + pos));
+          } else if constexpr (KIND == SHIFT_Y) {
+            z = ldf2<CG>(fin + (size_t)pos * N + line0);
+          } else if constexpr (KIND == ROT_P1) {
+            z = load_rot90_pair<CG, decltype(pair)::value>(fin, N, q, line0, pos);
+          } else if constexpr (KIND == ROT_P2) {
+            z = ldf2<CG>(fin + (size_t)pos * M + line0);
+          } else {
+            z = make_float2(ldf<CG>(fin + (size_t)line0 * M + pos), ldf<CG>(fin + (size_t)(line0 + 1) * M + pos));
+          }
+          if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
         }
-        if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
+        v[m] = z;
       }
-      v[m] = z;
-    }
+    };
+    if (KIND == ROT_P1 && !aligned(fin, 8)) load(std::false_type{});
+    else load(std::true_type{});
     if constexpr (KIND == SHIFT_X || KIND == ROT_P1) {
       if (bad) atomicOr(a.status, STATUS_NONFINITE);
     }
@@ -891,7 +897,8 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
         } else if constexpr (KIND == SHIFT_Y) {
           z = *reinterpret_cast<const float2 *>(fin + (size_t)pos * N + line0);
         } else if constexpr (KIND == ROT_P1) {
-          z = load_rot90_pair(fin, N, q, line0, pos);
+          z = aligned(fin, 8) ? load_rot90_pair(fin, N, q, line0, pos)
+                              : load_rot90_pair<false, false>(fin, N, q, line0, pos);
         }
       }
       if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
@@ -937,7 +944,7 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
   //   q = 1: element pos >= 1 of lines col0 + j is frame[n - pos][col0 + j];
   //   q = 3: element pos of line i >= 1 is frame[pos][n - i], i.e. columns
   //          n - col0 - 7 .. n - col0 for the CTA's lines col0 .. col0 + 7.
-  const bool RCOLS = (KIND == ROT_P1) && (q & 1);
+  const bool RCOLS = (KIND == ROT_P1) && (q & 1) && aligned(fin, 16);
   if (RCOLS) {
     if (q == 1) {
       constexpr int IT = HP * N / (32 * PPC);
@@ -993,7 +1000,8 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
     // one branch per line pair, not per element, so that each form's loads
     // are issued together: staged columns (odd quarter turns), rows (q = 0)
     // or rows read backwards (q = 2: element pos >= 1 of line i >= 1 is
-    // frame[n - i][n - pos])
+    // frame[n - i][n - pos]); column by column where the frame is not aligned
+    // for staging
     if (RCOLS) {
 #pragma unroll
       for (int m = 0; m < 32; m++) v[m] = (32 * m < NIN) ? buf[pad32(lane + 32 * m)] : make_float2(0.f, 0.f);
@@ -1004,6 +1012,10 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
         v[m] = (32 * m < NIN) ? make_float2(fin[(size_t)line0 * N + pos], fin[(size_t)(line0 + 1) * N + pos])
                               : make_float2(0.f, 0.f);
       }
+    } else if (q & 1) {
+#pragma unroll
+      for (int m = 0; m < 32; m++)
+        v[m] = (32 * m < NIN) ? load_rot90_pair<false, false>(fin, N, q, line0, lane + 32 * m) : make_float2(0.f, 0.f);
     } else {
       const float *r0 = fin + (size_t)(N - line0) * N + N;        // row n - line0 (unused for line0 = 0), + n
       const float *r1 = fin + (size_t)(N - line0 - 1) * N + N;    // row n - line0 - 1, + n

@@ -82,7 +82,9 @@ __device__ __forceinline__ float2 ldf2(const float *p) {
 }
 
 // Load element `pos` (< n) of row `line` of rot90^q(frame) and of row line+1.
-template <bool CG = false>
+// PAIR: the frame is 8-byte aligned (line is even), so that two adjacent
+// columns come in one load.
+template <bool CG = false, bool PAIR = true>
 __device__ __forceinline__ float2 load_rot90_pair(const float *__restrict__ fr, int n, int q, int line, int pos) {
   float x0 = 0.f, x1 = 0.f;
   switch (q) {
@@ -92,9 +94,15 @@ __device__ __forceinline__ float2 load_rot90_pair(const float *__restrict__ fr, 
       break;
     case 1:   // g[i][j] = in[n - j][i]  (j >= 1)
       if (pos >= 1) {
-        float2 t = ldf2<CG>(fr + (size_t)(n - pos) * n + line);
-        x0 = t.x;
-        x1 = t.y;
+        const float *p = fr + (size_t)(n - pos) * n + line;
+        if constexpr (PAIR) {
+          const float2 t = ldf2<CG>(p);
+          x0 = t.x;
+          x1 = t.y;
+        } else {
+          x0 = ldf<CG>(p);
+          x1 = ldf<CG>(p + 1);
+        }
       }
       break;
     case 2:   // g[i][j] = in[n - i][n - j]  (i, j >= 1)
@@ -110,6 +118,12 @@ __device__ __forceinline__ float2 load_rot90_pair(const float *__restrict__ fr, 
   }
   return make_float2(x0, x1);
 }
+
+// The frames of rotation pass 1 are the caller's: the allocation-free
+// rotation takes them at any float address (every other frame of the library
+// is 16-byte aligned, and so are the scratch frames).  The frame stride is a
+// multiple of 16 bytes, so all frames of a launch take the same form.
+__device__ __forceinline__ bool aligned(const float *p, int bytes) { return ((uintptr_t)p & (bytes - 1)) == 0; }
 
 }  // namespace
 }  // namespace graphic
