@@ -154,9 +154,13 @@ __global__ void __launch_bounds__(RANK_THREADS) full_rank_kernel(const GeneralAr
         }
       }
     }
-    bool bad = false;   // any of the segment's pixels
+    // the unit's own pixels, and those of the segment that no unit has (they
+    // are set to zero, or are the band path's, after every unit): other
+    // annuli's are their own units' to test, and in a call in place they may
+    // hold residuals by now
+    bool bad = false;
 #pragma unroll
-    for (int q = 0; q < SEG; q++) bad |= !(acc[q] == 0.f);
+    for (int q = 0; q < SEG; q++) bad |= !(acc[q] == 0.f) && (ann_s[q] == ann || ann_s[q] < 0);
     if (__any_sync(FULL, bad) && lane == 0) atomicOr(a.status, STATUS_NONFINITE);
   }
   __syncthreads();
@@ -542,7 +546,8 @@ __global__ void __launch_bounds__(512, 2) psf_sweep_kernel(const GeneralArgs g) 
 }
 
 // Pixels of no annulus in the general path's 4-pixel groups: residual 0 in
-// every frame.  One CTA per listed segment.
+// every frame, after the units, whose ranking tests these pixels' input (a
+// call may be in place).  One CTA per listed segment.
 __global__ void __launch_bounds__(128) general_zero_kernel(const AdiArgs a) {
   const long long p = (long long)__ldg(&a.zero[blockIdx.x]) * SEG + (threadIdx.x & (SEG - 1));
   if (annulus_of(p, a.n, a.iedge2, a.n_ann) >= 0 || !group_general(a, p)) return;
@@ -632,12 +637,13 @@ namespace {
 cudaError_t launch_adi_general(const AdiArgs &a, cudaStream_t st, int &nl) {
   const int T = a.T;
   cudaError_t e;
-  if (a.n_zero > 0) {
+  auto zero = [&]() {
+    if (a.n_zero == 0) return cudaSuccess;
     general_zero_kernel<<<(unsigned)a.n_zero, 128, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     nl++;
-  }
-  if (a.n_units == 0) return cudaSuccess;
+    return cudaGetLastError();
+  };
+  if (a.n_units == 0) return zero();
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
@@ -682,7 +688,7 @@ cudaError_t launch_adi_general(const AdiArgs &a, cudaStream_t st, int &nl) {
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     nl += 2;
   }
-  return cudaSuccess;
+  return zero();
 }
 
 }  // namespace
