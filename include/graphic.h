@@ -252,7 +252,7 @@ int graphic_sky_subtract(graphic_ctx *ctx, const float *in, float *out, int64_t 
  * of the n x n values of ref (FP64), the median by the rule above (FP32),
  * the comparison in FP64; else 0.  ref (a master dark or sky) and map
  * (uint8, n x n) are device buffers.  GRAPHIC_ERR_NONFINITE if ref holds a
- * non-finite value.
+ * non-finite value (map is then left as it was).
  */
 int graphic_bad_pixel_map(graphic_ctx *ctx, const float *ref, int32_t n, double C, uint8_t *map);
 

@@ -242,9 +242,10 @@ cudaError_t launch_sky_median(const CollapseArgs &a, cudaStream_t st);
 cudaError_t launch_sky_subtract(const float *in, float *out, long long T, int n, const float *skies,
                                 const int *sky_of_frame, cudaStream_t st);
 // bad pixel map of the n_vals values of ref, in a device workspace of
-// bad_map_bytes(): FP64 sums, the exact median by three 11-bit digits of the
-// total-order keys, then the map; all on the stream, no host step between
-// (result: the first double of the workspace is the sum of the values)
+// bad_map_bytes(): FP64 sums, the exact median by three digits (11, 11 and 10
+// bits) of the total-order keys, then the map; all on the stream, no host step
+// between (result: the first double of the workspace is the sum of the values;
+// where it is not finite the map is not written)
 size_t bad_map_bytes();
 cudaError_t launch_bad_map(const float *ref, long long n_vals, double C, uint8_t *map, void *ws, cudaStream_t st);
 // bad pixel correction: the flagged and non-finite pixels become NaN and are

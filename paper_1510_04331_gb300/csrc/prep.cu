@@ -160,9 +160,11 @@ __global__ void __launch_bounds__(MAP_THREADS) map_digit_kernel(const float *__r
 }
 
 // map[p] = |ref[p] - median| > C sigma (FP64 comparison; the median FP32: the
-// lower middle value, or the mean of the two for an even count).
+// lower middle value, or the mean of the two for an even count).  A frame
+// whose sum is not finite is refused by the caller: its map stays as it is.
 __global__ void __launch_bounds__(MAP_THREADS) bad_map_kernel(const float *__restrict__ ref, long long n, double C,
                                                               const MapWs *ws, uint8_t *map) {
+  if (!isfinite(ws->sums[0])) return;
   uint32_t key[2];
   map_prefix<3>(ws, n, key);
   auto val = [](uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k); };
