@@ -45,37 +45,41 @@ __global__ void sky_subtract_kernel(const float4 *__restrict__ in, float4 *__res
 // 250 us in all.
 constexpr int MAP_THREADS = 512;
 constexpr int MAP_BINS = 2048;
+// Count: 32 bits, 64 for frames of 2^32 pixels and more (64 bits everywhere
+// cost 5 us a call, in clearing and in reading twice the bytes per block).
+template <class Count>
 struct MapWs {
-  double sums[2];                      // sum, sum of squared deviations
-  unsigned int hist[3][2][MAP_BINS];   // [digit][lower, upper median]
+  double sums[2];               // sum, sum of squared deviations
+  Count hist[3][2][MAP_BINS];   // [digit][lower, upper median]
 };
 
 // Bin of rank k in a histogram of MAP_BINS global counts and the counts
 // before it, found by the whole block (each thread sums MAP_BINS /
 // MAP_THREADS bins, then a block scan); every thread gets the result.
-__device__ __forceinline__ void map_find(const unsigned int *hist, unsigned long long k, int &bin,
+template <class Count>
+__device__ __forceinline__ void map_find(const Count *hist, unsigned long long k, int &bin,
                                          unsigned long long &before) {
-  __shared__ unsigned int wsum[MAP_THREADS / 32];
+  __shared__ Count wsum[MAP_THREADS / 32];
   __shared__ int bin_s;
-  __shared__ unsigned int before_s;
+  __shared__ Count before_s;
   constexpr int PER = MAP_BINS / MAP_THREADS;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  unsigned int h[PER], s = 0;
+  Count h[PER], s = 0;
 #pragma unroll
   for (int b = 0; b < PER; b++) {
     h[b] = hist[threadIdx.x * PER + b];
     s += h[b];
   }
-  unsigned int inc = s;
+  Count inc = s;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const unsigned int t = __shfl_up_sync(0xffffffffu, inc, o);
+    const Count t = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += t;
   }
   __syncthreads();   // the shared words of an earlier call have been read
   if (lane == 31) wsum[w] = inc;
   __syncthreads();
-  unsigned int acc = inc - s;
+  Count acc = inc - s;
   for (int q = 0; q < w; q++) acc += wsum[q];
 #pragma unroll
   for (int b = 0; b < PER; b++) {
@@ -92,8 +96,8 @@ __device__ __forceinline__ void map_find(const unsigned int *hist, unsigned long
 
 // The key prefixes (aligned to bit 31) of the lower and upper median after
 // DIGITS digits, and the ranks left within them.
-template <int DIGITS>
-__device__ __forceinline__ void map_prefix(const MapWs *ws, long long n, uint32_t (&prefix)[2]) {
+template <int DIGITS, class Count>
+__device__ __forceinline__ void map_prefix(const MapWs<Count> *ws, long long n, uint32_t (&prefix)[2]) {
   unsigned long long k[2] = {(unsigned long long)((n - 1) / 2), (unsigned long long)(n / 2)};
   prefix[0] = prefix[1] = 0u;
 #pragma unroll
@@ -126,8 +130,9 @@ __device__ __forceinline__ void block_add(double acc, double *dst) {
 
 // Digit DIGIT's histograms of the keys that match the digits before it; with
 // the sum (DIGIT 0) or the squared deviations from the mean (DIGIT 1).
-template <int DIGIT>
-__global__ void __launch_bounds__(MAP_THREADS) map_digit_kernel(const float *__restrict__ v, long long n, MapWs *ws) {
+template <int DIGIT, class Count>
+__global__ void __launch_bounds__(MAP_THREADS) map_digit_kernel(const float *__restrict__ v, long long n,
+                                                                MapWs<Count> *ws) {
   __shared__ unsigned int h[2][MAP_BINS];
   for (int b = threadIdx.x; b < 2 * MAP_BINS; b += MAP_THREADS) h[b / MAP_BINS][b % MAP_BINS] = 0u;
   uint32_t prefix[2];
@@ -154,7 +159,7 @@ __global__ void __launch_bounds__(MAP_THREADS) map_digit_kernel(const float *__r
   __syncthreads();
   for (int b = threadIdx.x; b < 2 * MAP_BINS; b += MAP_THREADS) {
     const unsigned int c = h[b / MAP_BINS][b % MAP_BINS];
-    if (c) atomicAdd(&ws->hist[DIGIT][b / MAP_BINS][b % MAP_BINS], c);
+    if (c) atomicAdd(&ws->hist[DIGIT][b / MAP_BINS][b % MAP_BINS], (Count)c);
   }
   if constexpr (DIGIT < 2) block_add(acc, &ws->sums[DIGIT]);
 }
@@ -162,8 +167,9 @@ __global__ void __launch_bounds__(MAP_THREADS) map_digit_kernel(const float *__r
 // map[p] = |ref[p] - median| > C sigma (FP64 comparison; the median FP32: the
 // lower middle value, or the mean of the two for an even count).  A frame
 // whose sum is not finite is refused by the caller: its map stays as it is.
+template <class Count>
 __global__ void __launch_bounds__(MAP_THREADS) bad_map_kernel(const float *__restrict__ ref, long long n, double C,
-                                                              const MapWs *ws, uint8_t *map) {
+                                                              const MapWs<Count> *ws, uint8_t *map) {
   if (!isfinite(ws->sums[0])) return;
   uint32_t key[2];
   map_prefix<3>(ws, n, key);
@@ -367,6 +373,21 @@ unsigned grid_for(long long work, int threads) {
   return (unsigned)g;
 }
 
+template <class Count>
+cudaError_t bad_map(const float *ref, long long n_vals, double C, uint8_t *map, void *ws, cudaStream_t st) {
+  MapWs<Count> *w = static_cast<MapWs<Count> *>(ws);
+  cudaError_t e = cudaMemsetAsync(w, 0, sizeof(*w), st);
+  if (e != cudaSuccess) return e;
+  // at most one block per SM: each flushes its own histograms
+  long long grid = (n_vals + MAP_THREADS - 1) / MAP_THREADS;
+  if (grid > 152) grid = 152;
+  map_digit_kernel<0><<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, w);
+  map_digit_kernel<1><<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, w);
+  map_digit_kernel<2><<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, w);
+  bad_map_kernel<<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, C, w, map);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_sky_subtract(const float *in, float *out, long long T, int n, const float *skies,
@@ -379,20 +400,11 @@ cudaError_t launch_sky_subtract(const float *in, float *out, long long T, int n,
   return cudaGetLastError();
 }
 
-size_t bad_map_bytes() { return sizeof(MapWs); }
+size_t bad_map_bytes() { return sizeof(MapWs<unsigned long long>); }
 
 cudaError_t launch_bad_map(const float *ref, long long n_vals, double C, uint8_t *map, void *ws, cudaStream_t st) {
-  MapWs *w = static_cast<MapWs *>(ws);
-  cudaError_t e = cudaMemsetAsync(w, 0, sizeof(MapWs), st);
-  if (e != cudaSuccess) return e;
-  // at most one block per SM: each flushes its own histograms
-  long long grid = (n_vals + MAP_THREADS - 1) / MAP_THREADS;
-  if (grid > 152) grid = 152;
-  map_digit_kernel<0><<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, w);
-  map_digit_kernel<1><<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, w);
-  map_digit_kernel<2><<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, w);
-  bad_map_kernel<<<(unsigned)grid, MAP_THREADS, 0, st>>>(ref, n_vals, C, w, map);
-  return cudaGetLastError();
+  return n_vals < (1ll << 32) ? bad_map<unsigned int>(ref, n_vals, C, map, ws, st)
+                              : bad_map<unsigned long long>(ref, n_vals, C, map, ws, st);
 }
 
 size_t fix_count_words(long long T) { return 2 + (size_t)T; }

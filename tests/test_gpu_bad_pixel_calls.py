@@ -29,3 +29,29 @@ def test_map_of_a_refused_frame_is_left_alone(g, n, value):
     rc = g.lib().graphic_bad_pixel_map(ctx.h, ctypes.c_void_p(ref.data_ptr()), n, 2.0, ctypes.c_void_p(bad.data_ptr()))
     assert rc == -5, rc
     assert bool((bad == 7).all())
+
+
+def _room(gib):
+    if torch.cuda.mem_get_info()[0] < gib * 2 ** 30:
+        pytest.skip(f"needs {gib} GiB of device memory")
+
+
+@pytest.mark.parametrize("case", ["one bin", "ramp"])
+def test_map_of_frames_beyond_32_bit_counts(g, case):
+    """One bin that holds more than 2^32 pixels; a ramp with more than 2^32 pixels in the bins below the middle's."""
+    _room(60)
+    if case == "one bin":
+        n = 65600
+        ref = torch.full((n, n), 2.5, device="cuda")
+        ref[5] = 3.5
+        want = np.arange(n) == 5
+    else:
+        n = 100000
+        ref = torch.arange(n, dtype=torch.float32, device="cuda")[:, None].expand(n, n).contiguous()
+        # n values of each row number: median (n - 1) / 2, sigma sqrt((n^2 - 1) / 12)
+        want = np.abs(np.arange(n) - (n - 1) / 2) > np.sqrt((n * n - 1.0) / 12.0)
+    got = g.context().graphic_bad_pixel_map(ref, 1.0)
+    lo, hi = got.amin(dim=1).cpu().numpy(), got.amax(dim=1).cpu().numpy()
+    assert np.array_equal(lo, want) and np.array_equal(hi, want)
+    del ref, got
+    torch.cuda.empty_cache()
