@@ -197,7 +197,8 @@ __device__ __forceinline__ void count_block(unsigned long long mine, unsigned lo
 
 // Flagged and non-finite pixels become NaN, are counted per frame and, up to
 // `cap` a frame, listed: pixel p of frame f as list[f nn + j], j from the
-// frame's counter (any order).  One block per (chunk of MARK_CHUNK pixels, frame): four values and four map bytes
+// frame's counter (any order).  Without lists (cap 0) the count only says
+// whether there is one: a frame may hold 2^32 pixels.  One block per (chunk of MARK_CHUNK pixels, frame): four values and four map bytes
 // per load where frames and map are aligned for it (VEC), no division per
 // value.  HBM-bound: 200 frames of 512 x 512 in 52 us = 4.0 TB/s, against 207
 // us with a 64-bit modulo and 4-byte accesses per value.  The fill of the
@@ -219,6 +220,10 @@ __global__ void __launch_bounds__(MARK_THREADS) bad_mark_kernel(float *__restric
     uint32_t *lf = list + f * nn, *cnt = counts + f;
     auto add = [&](long long p) {
       fr[p] = NANF;
+      if (cap == 0) {
+        atomicOr(cnt, 1u);
+        return;
+      }
       const uint32_t j = atomicAdd(cnt, 1u);
       if (j < cap) lf[j] = (uint32_t)p;
     };

@@ -55,3 +55,23 @@ def test_map_of_frames_beyond_32_bit_counts(g, case):
     assert np.array_equal(lo, want) and np.array_equal(hi, want)
     del ref, got
     torch.cuda.empty_cache()
+
+
+def test_correction_of_a_frame_of_2_32_bad_pixels(g):
+    _room(60)
+    n = 65536
+    ctx = g.Context(torch.cuda.current_device())   # its scratch, as large as the frame, goes with it
+    try:
+        x = torch.full((1, n, n), float("nan"), device="cuda")
+        ctx._stream()
+        rc = g.lib().graphic_bad_pixel_fix(ctx.h, ctypes.c_void_p(x.data_ptr()), 1, n, None)
+        assert rc == -5, rc
+        x.fill_(2.0)
+        x[0, 7, 9] = float("inf")
+        rc = g.lib().graphic_bad_pixel_fix(ctx.h, ctypes.c_void_p(x.data_ptr()), 1, n, None)
+        assert rc == 0, rc
+        assert bool((x == 2.0).all())
+        del x
+    finally:
+        ctx.close()
+    torch.cuda.empty_cache()
