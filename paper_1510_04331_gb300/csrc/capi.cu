@@ -37,7 +37,7 @@ struct graphic_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   int *d_status = nullptr;
-  int *h_status = nullptr;          // pinned: the status word, then 8 bytes of results read back by a call
+  int *h_status = nullptr;          // pinned: the status word, then from word 2 on 16 bytes of results read back by a call
   char *d_plan = nullptr;
   size_t d_plan_bytes = 0;
   char *h_plan = nullptr;           // pinned staging
@@ -1351,7 +1351,7 @@ int graphic_create(graphic_ctx **out, int device) {
     return fail(GRAPHIC_ERR_CUDA, "twiddle table upload failed");
   }
   e = cudaMalloc(&c->d_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost(&c->h_status, 4 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost(&c->h_status, 8 * sizeof(int));
   if (e != cudaSuccess) {
     graphic_destroy(c);
     return cuda_fail(e, "context allocation");
@@ -1854,23 +1854,30 @@ int graphic_bad_pixel_fix(graphic_ctx *c, float *cube, int64_t T, int32_t n, con
   const uint32_t counts[2] = {(uint32_t)c->h_status[2], (uint32_t)c->h_status[3]};
   bool hopeless = counts[1] > 0;
   if (counts[0] > 0) {
-    // frames with more pixels to fill than a list holds: dense passes
-    // between the cube and the scratch, over every frame (the others hold no
-    // NaN any more)
-    unsigned long long *d_cnt = reinterpret_cast<unsigned long long *>(c->d_prep + 2048);   // [2]
-    unsigned long long cnt[2] = {1, 1};   // NaN left, filled
+    // frames with more pixels to fill than a list takes: dense passes over
+    // those frames, between the cube and the scratch; a pair of counters (NaN
+    // left, filled) a pass, cleared SLOTS passes at a time
+    constexpr int SLOTS = 2048 / 16;
+    unsigned long long *d_cnt = reinterpret_cast<unsigned long long *>(c->d_prep + 2048);   // [SLOTS][2]
+    const uint32_t *frames = counts[0] == T ? nullptr : d_counts + 2 + T;
+    unsigned long long *cnt = reinterpret_cast<unsigned long long *>(c->h_status + 2);
+    cnt[0] = cnt[1] = 1;
     float *src = cube, *dst = c->d_scratch;
     for (int pass = 0; cnt[0] > 0 && cnt[1] > 0 && pass <= 2 * n; pass++) {
-      CK(cudaMemsetAsync(d_cnt, 0, sizeof(cnt), c->stream));
-      e = launch_bad_pass(src, dst, T, n, d_cnt, c->stream);
+      unsigned long long *slot = d_cnt + 2 * (pass % SLOTS);
+      if (pass % SLOTS == 0) CK(cudaMemsetAsync(d_cnt, 0, SLOTS * 16, c->stream));
+      e = launch_bad_pass(src, dst, counts[0], n, frames, slot, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "bad pixel pass kernel");
-      CK(cudaMemcpyAsync(cnt, d_cnt, sizeof(cnt), cudaMemcpyDeviceToHost, c->stream));
+      CK(cudaMemcpyAsync(cnt, slot, 16, cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
       std::swap(src, dst);
     }
     hopeless |= cnt[0] > 0;
     if (src != cube) {
-      CK(cudaMemcpyAsync(cube, src, bytes, cudaMemcpyDeviceToDevice, c->stream));
+      // a pass with nothing more to fill copies the listed frames
+      e = frames ? launch_bad_pass(src, cube, counts[0], n, frames, d_cnt, c->stream)
+                 : cudaMemcpyAsync(cube, src, bytes, cudaMemcpyDeviceToDevice, c->stream);
+      if (e != cudaSuccess) return cuda_fail(e, "bad pixel copy");
       CK(cudaStreamSynchronize(c->stream));
     }
   }

@@ -249,17 +249,19 @@ cudaError_t launch_sky_subtract(const float *in, float *out, long long T, int n,
 size_t bad_map_bytes();
 cudaError_t launch_bad_map(const float *ref, long long n_vals, double C, uint8_t *map, void *ws, cudaStream_t st);
 // bad pixel correction: the flagged and non-finite pixels become NaN and are
-// listed per frame (ws: n x n words a frame), then each frame with at most
-// n x n / 2 of them (n <= 65535) is filled from its list.  counts (device, fix_count_words(T)
-// u32): [0] frames with more (left to the dense passes), [1] pixels of other
-// frames that no pass can fill, [2..2+T) listed pixels
+// listed per frame (ws: n x n words a frame), then each frame with few enough
+// of them (prep.cu, list_cap) is filled from its list.  counts (device,
+// fix_count_words(T) u32): [0] frames with more, left to the dense passes, [1]
+// pixels of other frames that no pass can fill, [2..2+T) marked pixels per
+// frame, [2+T...) the frames left
 size_t fix_count_words(long long T);
 cudaError_t launch_bad_fill(float *cube, long long T, int n, const uint8_t *map, uint32_t *ws, uint32_t *counts,
                             cudaStream_t st);
-// one dense pass: every NaN pixel of src with a finite 8-neighbour filled
-// into dst, the others copied; counts[0] += NaN left, counts[1] += filled
-cudaError_t launch_bad_pass(const float *src, float *dst, long long T, int n, unsigned long long *counts,
-                            cudaStream_t st);
+// one dense pass over the D frames listed in `frames` (device; null: frames
+// 0 .. D - 1): every NaN pixel of src with a finite 8-neighbour filled into dst, the others copied;
+// counts[0] += NaN left, counts[1] += filled
+cudaError_t launch_bad_pass(const float *src, float *dst, uint32_t D, int n, const uint32_t *frames,
+                            unsigned long long *counts, cudaStream_t st);
 
 // register.cu: registration (Sect. 3.1), one CTA per frame
 struct RegArgs {

@@ -198,12 +198,13 @@ __device__ __forceinline__ void count_block(unsigned long long mine, unsigned lo
 // Flagged and non-finite pixels become NaN, are counted per frame and, up to
 // `cap` a frame, listed: pixel p of frame f as list[f nn + j], j from the
 // frame's counter (any order).  Without lists (cap 0) the count only says
-// whether there is one: a frame may hold 2^32 pixels.  One block per (chunk of MARK_CHUNK pixels, frame): four values and four map bytes
-// per load where frames and map are aligned for it (VEC), no division per
-// value.  HBM-bound: 200 frames of 512 x 512 in 52 us = 4.0 TB/s, against 207
-// us with a 64-bit modulo and 4-byte accesses per value.  The fill of the
-// 0.1 % listed pixels takes 19 us, where two dense passes over the cube took
-// 331.
+// whether there is one: a frame may hold 2^32 pixels.  One block per (chunk of
+// MARK_CHUNK pixels, frame): four values and four map bytes per load where
+// frames and map are aligned for it (VEC), no division per value; a warp's
+// marked pixels take their places with one step of the counter (a step per
+// pixel: 200 frames of 512 x 512 with 5 % bad 1526 us a call, 220 so).
+// HBM-bound where little is marked: 200 frames of 512 x 512 in 52 us = 4.0
+// TB/s, against 207 us with a 64-bit modulo and 4-byte accesses per value.
 constexpr int MARK_THREADS = 256;
 constexpr int MARK_CHUNK = MARK_THREADS * 16;
 template <bool VEC>
@@ -213,19 +214,25 @@ __global__ void __launch_bounds__(MARK_THREADS) bad_mark_kernel(float *__restric
                                                                 uint32_t *__restrict__ list, uint32_t *counts) {
   const float NANF = __uint_as_float(0x7fc00000u);
   const long long items = T * chunks;
+  const int lane = threadIdx.x & 31;
   for (long long it = blockIdx.x; it < items; it += gridDim.x) {
     const long long f = it / chunks;
     const long long c0 = (it - f * chunks) * MARK_CHUNK;
     float *fr = cube + f * nn;
     uint32_t *lf = list + f * nn, *cnt = counts + f;
-    auto add = [&](long long p) {
-      fr[p] = NANF;
-      if (cap == 0) {
-        atomicOr(cnt, 1u);
-        return;
+    // count and list the warp's marked pixels: bit b of a lane's m is pixel at(b)
+    auto add = [&](uint32_t m, auto at) {
+      if (!__any_sync(0xffffffffu, m != 0u)) return;
+      const uint32_t mine = __popc(m);
+      uint32_t end = mine, j = 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += t;
       }
-      const uint32_t j = atomicAdd(cnt, 1u);
-      if (j < cap) lf[j] = (uint32_t)p;
+      if (lane == 31) j = cap > 0 ? atomicAdd(cnt, end) : atomicOr(cnt, 1u);
+      j = __shfl_sync(0xffffffffu, j, 31) + end - mine;
+      for (; m && j < cap; m &= m - 1, j++) lf[j] = (uint32_t)at(__ffs(m) - 1);
     };
     if constexpr (VEC) {
       float4 v[4];
@@ -236,19 +243,30 @@ __global__ void __launch_bounds__(MARK_THREADS) bad_mark_kernel(float *__restric
         v[k] = p < nn ? __ldcs(reinterpret_cast<const float4 *>(fr + p)) : make_float4(0.f, 0.f, 0.f, 0.f);
         b[k] = p < nn && map ? __ldg(reinterpret_cast<const uint32_t *>(map + p)) : 0u;
       }
+      uint32_t m = 0u;
 #pragma unroll
       for (int k = 0; k < 4; k++) {
-        const long long p = c0 + 4 * (threadIdx.x + k * MARK_THREADS);
-        const bool fin = isfinite(v[k].x) && isfinite(v[k].y) && isfinite(v[k].z) && isfinite(v[k].w);
-        if (fin && b[k] == 0u) continue;
-        const float q[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+        float q[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+        uint32_t mk = 0u;
 #pragma unroll
         for (int l = 0; l < 4; l++)
-          if (!isfinite(q[l]) || ((b[k] >> (8 * l)) & 255u)) add(p + l);
+          if (!isfinite(q[l]) || ((b[k] >> (8 * l)) & 255u)) {
+            q[l] = NANF;
+            mk |= 1u << l;
+          }
+        if (mk)
+          *reinterpret_cast<float4 *>(fr + c0 + 4 * (threadIdx.x + k * MARK_THREADS)) =
+              make_float4(q[0], q[1], q[2], q[3]);
+        m |= mk << (4 * k);
       }
+      add(m, [&](int i) { return c0 + 4 * (threadIdx.x + (i >> 2) * MARK_THREADS) + (i & 3); });
     } else {
-      for (long long p = c0 + threadIdx.x; p < min(nn, c0 + MARK_CHUNK); p += MARK_THREADS)
-        if (!isfinite(fr[p]) || (map && map[p])) add(p);
+      for (long long q0 = c0; q0 < min(nn, c0 + MARK_CHUNK); q0 += MARK_THREADS) {
+        const long long p = q0 + threadIdx.x;
+        const bool bad = p < nn && (!isfinite(fr[p]) || (map && map[p]));
+        if (bad) fr[p] = NANF;
+        add(bad ? 1u : 0u, [&](int) { return p; });
+      }
     }
   }
 }
@@ -285,26 +303,56 @@ __device__ __forceinline__ bool neighbour_median(const float *fr, int n, int r, 
   return true;
 }
 
+// Most pixels a frame's list may hold where D frames hold more than a short
+// list (D = 1).  A pass over a list costs its frame a round of one block per
+// 1024 pixels left, whatever the other frames do; a dense pass costs every
+// pixel of the D frames, but all blocks share it.  Calls with 1024 threads a
+// frame, listed and dense (calls in dense passes only): one frame of 512 x 512
+// with 1310 bad pixels 46 us (75), with 2621 57 (79); of 1024 x 1024 with 5243 70
+// (83), with 10 486 93 (85); eight of 512 x 512 with 13 107 each 98 (119), with
+// 26 214 156 (121); 50 of 1024 x 1024 with 104 858 702 (922), with 209 715 1184
+// (1060); 200 of 512 x 512 with 104 858 890 (1411).  Lists of up to half a frame,
+// whatever D: one frame of 1024 x 1024 with 40 % bad 5441 us, 107 so.
+// List and fill values share a frame's n x n words, pixel numbers have 32 bits.
+__host__ __device__ inline uint32_t list_cap(long long D, long long nn) {
+  if (nn >= (1ll << 32)) return 0u;
+  const long long half = nn / 2, c = 4096 + D * nn / 320;
+  return (uint32_t)(c < half ? c : half);
+}
+
 // One block per frame fills the frame's listed pixels pass by pass: every
 // pixel of a pass reads the values of the pass before (a pass keeps its fills
 // in vals and writes them after a barrier), filled pixels leave the list,
 // until it is empty or a pass fills nothing.  A pass costs the pixels left,
-// not the frame.  Frames with more than `cap` pixels to fill are counted and
-// left to the dense passes.
-constexpr int FILL_THREADS = 256;
+// not the frame.  Frames with too many pixels for that are listed in
+// counts[2 + T ...] and left to the dense passes.  `cap`: the lists' room.
+template <int FILL_THREADS>
 __global__ void __launch_bounds__(FILL_THREADS) bad_fill_kernel(float *cube, long long T, int n, uint32_t cap,
                                                                 uint32_t *lists, uint32_t *counts) {
   const long long nn = (long long)n * n;
   const float NANF = __uint_as_float(0x7fc00000u);
-  __shared__ uint32_t kept_s;
+  const uint32_t few = list_cap(1, nn);
+  __shared__ uint32_t kept_s, many_s;
   for (long long f = blockIdx.x; f < T; f += gridDim.x) {
     float *fr = cube + f * nn;
     uint32_t *list = lists + f * nn;
     float *vals = reinterpret_cast<float *>(list + cap);   // cap + cap <= nn
     uint32_t left = counts[2 + f];
-    if (left > cap) {
-      if (threadIdx.x == 0) atomicAdd(&counts[0], 1u);
-      continue;
+    if (left > few) {
+      // the frames that would share the dense passes
+      if (threadIdx.x == 0) many_s = 0u;
+      __syncthreads();
+      uint32_t many = 0u;
+      for (long long t = threadIdx.x; t < T; t += FILL_THREADS) many += counts[2 + t] > few ? 1u : 0u;
+      many = __reduce_add_sync(0xffffffffu, many);
+      if ((threadIdx.x & 31) == 0) atomicAdd(&many_s, many);
+      __syncthreads();
+      many = many_s;
+      __syncthreads();
+      if (left > list_cap(many, nn)) {
+        if (threadIdx.x == 0) counts[2 + T + atomicAdd(&counts[0], 1u)] = (uint32_t)f;
+        continue;
+      }
     }
     while (left > 0) {
       for (uint32_t j = threadIdx.x; j < left; j += FILL_THREADS) {
@@ -341,31 +389,37 @@ __global__ void __launch_bounds__(FILL_THREADS) bad_fill_kernel(float *cube, lon
   }
 }
 
-// One pass: every NaN pixel with a finite 8-neighbour in src takes the median
-// of those neighbours (two middle values averaged for an even count, FP32);
-// counts[0] += NaN pixels left, counts[1] += pixels filled.
-__global__ void bad_pass_kernel(const float *__restrict__ src, float *__restrict__ dst, long long T, int n,
-                                unsigned long long *counts) {
+// One pass over the D frames listed in `frames` (null: frames 0 .. D - 1): every NaN pixel with a finite
+// 8-neighbour in src takes the median of those neighbours (two middle values
+// averaged for an even count, FP32), the others are copied; counts[0] += NaN
+// pixels left, counts[1] += pixels filled.  Blocks (pixels, frame).
+constexpr int PASS_THREADS = 256;
+__global__ void __launch_bounds__(PASS_THREADS) bad_pass_kernel(const float *__restrict__ src,
+                                                                float *__restrict__ dst, uint32_t D, int n,
+                                                                const uint32_t *__restrict__ frames,
+                                                                unsigned long long *counts) {
   unsigned long long left = 0, filled = 0;
-  const long long nn = (long long)n * n, total = T * nn;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float v = src[i];
-    if (!isnan(v)) {
-      dst[i] = v;
-      continue;
+  const long long nn = (long long)n * n;
+  for (uint32_t k = blockIdx.y; k < D; k += gridDim.y) {
+    const long long f = frames ? __ldg(&frames[k]) : k;
+    const float *s = src + f * nn;
+    float *d = dst + f * nn;
+    for (long long p = blockIdx.x * PASS_THREADS + threadIdx.x; p < nn; p += gridDim.x * PASS_THREADS) {
+      const float v = s[p];
+      if (!isnan(v)) {
+        d[p] = v;
+        continue;
+      }
+      const int r = (int)(p / n);
+      float med;
+      if (!neighbour_median(s, n, r, (int)(p - (long long)r * n), med)) {
+        d[p] = v;
+        left++;
+        continue;
+      }
+      d[p] = med;
+      filled++;
     }
-    const long long f = i / nn;
-    const long long p = i - f * nn;
-    const int r = (int)(p / n);
-    float med;
-    if (!neighbour_median(src + f * nn, n, r, (int)(p - (long long)r * n), med)) {
-      dst[i] = v;
-      left++;
-      continue;
-    }
-    dst[i] = med;
-    filled++;
   }
   count_block(left, &counts[0]);
   count_block(filled, &counts[1]);
@@ -412,15 +466,14 @@ cudaError_t launch_bad_map(const float *ref, long long n_vals, double C, uint8_t
                               : bad_map<unsigned long long>(ref, n_vals, C, map, ws, st);
 }
 
-size_t fix_count_words(long long T) { return 2 + (size_t)T; }
+size_t fix_count_words(long long T) { return 2 + 2 * (size_t)T; }
 
 cudaError_t launch_bad_fill(float *cube, long long T, int n, const uint8_t *map, uint32_t *ws, uint32_t *counts,
                             cudaStream_t st) {
   const long long nn = (long long)n * n;
   const long long chunks = (nn + MARK_CHUNK - 1) / MARK_CHUNK;
-  // list and fill values share a frame's n x n words; 32-bit pixel numbers
-  const uint32_t cap = nn < (1ll << 32) ? (uint32_t)(nn / 2) : 0u;
-  cudaError_t e = cudaMemsetAsync(counts, 0, fix_count_words(T) * sizeof(uint32_t), st);
+  const uint32_t cap = list_cap(T, nn);
+  cudaError_t e = cudaMemsetAsync(counts, 0, (2 + (size_t)T) * sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   const long long items = T * chunks;
   const unsigned grid = (unsigned)std::min<long long>(items, 152ll * 64);
@@ -429,14 +482,24 @@ cudaError_t launch_bad_fill(float *cube, long long T, int n, const uint8_t *map,
   else bad_mark_kernel<false><<<grid, MARK_THREADS, 0, st>>>(cube, T, nn, chunks, cap, map, ws, counts + 2);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  bad_fill_kernel<<<(unsigned)std::min<long long>(T, 1 << 20), FILL_THREADS, 0, st>>>(cube, T, n, cap, ws, counts);
+  // the widest blocks, that is the shortest chain per frame, of which every
+  // frame has one resident (2048 threads an SM); with more frames, which fill
+  // the chip by their number, 256 threads (2000 of 256 x 256 with 0.1 % bad 132
+  // us, 160 with 1024 threads; 310 of 1024 x 1024 with 40 % 8257, 5210 with 512)
+  const unsigned fills = (unsigned)std::min<long long>(T, 1 << 20);
+  if (T <= 304) bad_fill_kernel<1024><<<fills, 1024, 0, st>>>(cube, T, n, cap, ws, counts);
+  else if (T <= 608) bad_fill_kernel<512><<<fills, 512, 0, st>>>(cube, T, n, cap, ws, counts);
+  else bad_fill_kernel<256><<<fills, 256, 0, st>>>(cube, T, n, cap, ws, counts);
   return cudaGetLastError();
 }
 
-cudaError_t launch_bad_pass(const float *src, float *dst, long long T, int n, unsigned long long *counts,
-                            cudaStream_t st) {
+cudaError_t launch_bad_pass(const float *src, float *dst, uint32_t D, int n, const uint32_t *frames,
+                            unsigned long long *counts, cudaStream_t st) {
   const long long nn = (long long)n * n;
-  bad_pass_kernel<<<grid_for(T * nn, 256), 256, 0, st>>>(src, dst, T, n, counts);
+  // the chip's blocks twice over, at least one a frame
+  const unsigned gy = std::min(D, 65535u);
+  const unsigned gx = (unsigned)std::min<long long>((nn + PASS_THREADS - 1) / PASS_THREADS, (152 * 16 + gy - 1) / gy);
+  bad_pass_kernel<<<dim3(gx, gy), PASS_THREADS, 0, st>>>(src, dst, D, n, frames, counts);
   return cudaGetLastError();
 }
 

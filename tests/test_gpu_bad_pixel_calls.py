@@ -75,3 +75,46 @@ def test_correction_of_a_frame_of_2_32_bad_pixels(g):
     finally:
         ctx.close()
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("T,n,counts", [
+    # lists of up to 4096 + D n^2 / 320 pixels, D frames with more than 4096 + n^2 / 320
+    (3, 256, [4300, 4301, 5]), (3, 256, [4505, 4506, 5]),
+    (1, 512, [4915]), (1, 512, [4916]),
+    # half a frame; the fills of more than 304 and of more than 608 frames
+    (305, 64, [0, 1, 40, 2047, 2048, 2049, 3000, 4095]), (609, 64, [0, 1, 40, 2047, 2048, 2049, 3000, 4095]),
+])
+def test_correction_around_the_longest_list(g, T, n, counts):
+    rng = np.random.default_rng(T + n)
+    c = rng.normal(0, 1, (T, n, n)).astype(np.float32)
+    for t in range(T):
+        k = counts[t % len(counts)]
+        where = np.arange(k) if t % 2 else rng.choice(n * n, k, replace=False)   # a block of rows, or anywhere
+        c[t].ravel()[where] = np.nan
+    want, st = oracle.bad_pixel_fix(c, None)
+    assert st == 0
+    x = torch.from_numpy(c).cuda()
+    g.context().graphic_bad_pixel_fix(x)
+    assert np.array_equal(x.cpu().numpy(), want)
+
+
+def test_correction_of_a_frame_with_many_bad_pixels_uses_the_whole_chip(g):
+    """40 % bad pixels may take a few times as long as 0.1 % (more pixels, some more passes); a frame filled by one
+    block takes a hundred times as long."""
+    n = 1024
+    src = torch.randn((1, n, n), device="cuda")
+    u = torch.rand((1, n, n), device="cuda")
+    ms = []
+    for share in (0.001, 0.4):
+        bad = torch.where(u < share, torch.full_like(src, float("nan")), src)
+        best = 1e9
+        for _ in range(6):
+            x = bad.clone()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.context().graphic_bad_pixel_fix(x)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms.append(best)
+    assert ms[1] < 10 * ms[0], ms
