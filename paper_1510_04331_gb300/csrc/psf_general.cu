@@ -27,7 +27,7 @@
 // Before (one kernel, 8 pixels per CTA and one CTA per SM: a radix sort per
 // pixel, then queries across the lanes, each lane meeting its events at other
 // queries and walking its own words): 600 frames of 256 x 256 with a time
-// gate 3.61 ms, now 1.21 (ranking 0.48, sweep 0.73); 2000 frames of 128 x 128
+// gate 3.61 ms, so 1.21 (ranking 0.48, sweep 0.73); 2000 frames of 128 x 128
 // 2.86 ms.  Bound by instruction issue (65 %) and the codes' loads.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -634,6 +634,8 @@ size_t general_scratch_bytes(const AdiPlanHost &ap, int64_t T) {
 
 namespace {
 
+constexpr size_t kPlainSmem = 47 * 1024;   // dynamic shared memory that needs no attribute (48 KB with the static)
+
 cudaError_t launch_adi_general(const AdiArgs &a, cudaStream_t st, int &nl) {
   const int T = a.T;
   cudaError_t e;
@@ -659,26 +661,41 @@ cudaError_t launch_adi_general(const AdiArgs &a, cudaStream_t st, int &nl) {
   // frames' ties without the radix sort)
   void (*rank)(GeneralArgs) = T <= 256 ? full_rank_kernel<256> : full_rank_kernel<1024>;
   const size_t rsmem = SEG * (T <= 256 ? full_pixel_bytes<256>(T) : full_pixel_bytes<1024>(T));
-  if ((e = cudaFuncSetAttribute(rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem)) != cudaSuccess) return e;
+  if (rsmem > kPlainSmem &&
+      (e = cudaFuncSetAttribute(rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem)) != cudaSuccess)
+    return e;
   // sweep: chunks of at least 32 queries; of 16, 8 or 4 warps a CTA the most
   // that leaves the most warps resident (32 by registers: 2000 frames, whose
-  // maps take 9 KB a warp, 2.86 ms for 128 x 128 with 8 warps, 3.30 with 16);
-  // few units: more chunks until the SMs have 16 warps each
+  // maps take 9 KB a warp, 2.86 ms for 128 x 128 with 8 warps, 3.30 with 16)
   const size_t maps = sweep_warp_bytes(g.NB / 32);
   int warps = 16;
   auto resident = [&](int w) {
     return std::min<long long>(32 / w, per_sm / (long long)(w * maps + SWEEP_SINK + 1024)) * w;
   };
   while (warps > 4 && resident(warps / 2) > resident(warps)) warps /= 2;
+  const int most = warps;
   warps = std::min(warps, std::max(1, T / 32));
-  const size_t ssmem = SWEEP_SINK + warps * maps;
   int cols = 1;
   while ((T + warps * cols - 1) / (warps * cols) > 128 ||
          ((long long)per * warps * cols < 16ll * sms && T / (warps * cols * 2) >= 32))
     cols *= 2;
+  // few units leave SMs idle for as long as a chunk takes: chunks of down to 4
+  // queries (each builds its own map first) until the SMs have 24 warps each.
+  // Sweeps with chunks of 32 queries and 16 warps, then so: two annuli of 64 x
+  // 64, 64 frames 38 -> 8 us, 1000 frames 315 -> 53; all of 64 x 64, 2048 frames
+  // 1057 -> 772; the two inner annuli of 2000 x 512 x 512 125 -> 110 (16 warps
+  // 103, 32 140; 64 x 64 x 1000 329, 197 and 198)
+  const int chunks = (int)std::min<long long>((T + 3) / 4, (24ll * sms + per - 1) / per);
+  if (chunks > warps * cols) {
+    warps = std::min(most, chunks);
+    cols = (chunks + warps - 1) / warps;
+  }
+  const size_t ssmem = SWEEP_SINK + warps * maps;
   g.C = (T + warps * cols - 1) / (warps * cols);
   void (*sweep)(GeneralArgs) = a.perm_id ? psf_sweep_kernel<false> : psf_sweep_kernel<true>;
-  if ((e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem)) != cudaSuccess) return e;
+  if (ssmem > kPlainSmem &&
+      (e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem)) != cudaSuccess)
+    return e;
   for (int u0 = 0; u0 < a.n_units; u0 += per) {
     const unsigned nu = (unsigned)std::min(per, a.n_units - u0);
     g.units = a.units + (size_t)u0 * UNIT_SEGS;
