@@ -490,11 +490,7 @@ cudaError_t launch_sky_median(const CollapseArgs &a, cudaStream_t st) {
   // power of two from 64 on: whole blocks); longer stacks one warp per pixel
   if (a.T <= 64) {
     const unsigned blocks = (unsigned)(NN / 128);
-    if (a.T <= 8) sky_net_kernel<8><<<blocks, 128, 0, st>>>(a);
-    else if (a.T <= 16) sky_net_kernel<16><<<blocks, 128, 0, st>>>(a);
-    else if (a.T <= 32) sky_net_kernel<32><<<blocks, 128, 0, st>>>(a);
-    else if (a.T <= 50) sky_net_kernel<50><<<blocks, 128, 0, st>>>(a);
-    else sky_net_kernel<64><<<blocks, 128, 0, st>>>(a);
+    with_median_width((int)a.T, [&](auto w) { sky_net_kernel<decltype(w)::value><<<blocks, 128, 0, st>>>(a); });
     return cudaGetLastError();
   }
   const unsigned grid = (unsigned)(NN / COL_PPC);

@@ -163,24 +163,14 @@ cudaError_t bin_launch(const float *in, float *out, long long T, long long nn, l
 cudaError_t launch_median_network(const float *in, float *out, long long T, int n, long long fs, int B, int *status,
                                   cudaStream_t st) {
   const long long nn = (long long)n * n;
-  // the narrowest network that holds a bin (the comparators grow faster than
-  // W); two pixels per thread (8-byte loads) up to 32 values: 1000 frames of
-  // 512 x 512 in 165 us against 195 for B = 10, 185 / 194 for 32; from 40 on
-  // their registers cost more (B = 50: 240 us with one pixel, 260 with two)
-  if (B <= 2) return bin_launch<2, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 4) return bin_launch<4, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 6) return bin_launch<6, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 8) return bin_launch<8, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 10) return bin_launch<10, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 12) return bin_launch<12, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 16) return bin_launch<16, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 20) return bin_launch<20, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 24) return bin_launch<24, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 32) return bin_launch<32, 2>(in, out, T, nn, fs, B, status, st);
-  if (B <= 40) return bin_launch<40, 1>(in, out, T, nn, fs, B, status, st);
-  if (B <= 50) return bin_launch<50, 1>(in, out, T, nn, fs, B, status, st);
-  if (B <= 64) return bin_launch<64, 1>(in, out, T, nn, fs, B, status, st);
-  return cudaErrorInvalidValue;
+  if (B > 64) return cudaErrorInvalidValue;
+  // two pixels per thread (8-byte loads) up to 32 values: 1000 frames of 512 x
+  // 512 in 165 us against 195 for B = 10, 185 / 194 for 32; from 40 on their
+  // registers cost more (B = 50: 240 us with one pixel, 260 with two)
+  return with_median_width(B, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    return bin_launch<W, W <= 32 ? 2 : 1>(in, out, T, nn, fs, B, status, st);
+  });
 }
 
 cudaError_t launch_bin_median(const float *in, float *out, long long T, int n, int B, int *status, cudaStream_t st,

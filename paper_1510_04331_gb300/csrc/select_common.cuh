@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace graphic {
 namespace {
 
@@ -79,6 +81,28 @@ __device__ __forceinline__ void merge_exchange(float (&v)[W]) {
 template <int W>
 __device__ __forceinline__ void middle_pair(float (&v)[W]) {
   merge_exchange<W, 1, 1>(v);
+}
+
+// The network for m <= 64 values: f(std::integral_constant<int, W>) with the
+// narrowest W built that holds them (the comparators grow faster than W).  From
+// 6 on every width is at most a third more than the one before, so that no
+// stack pays for more than a third more slots than it has; 50 stands where the
+// steps would have 48, the longer bins of Sect. 4.3 being of 50 frames.
+template <class F>
+inline auto with_median_width(int m, F f) {
+  if (m <= 2) return f(std::integral_constant<int, 2>{});
+  if (m <= 4) return f(std::integral_constant<int, 4>{});
+  if (m <= 6) return f(std::integral_constant<int, 6>{});
+  if (m <= 8) return f(std::integral_constant<int, 8>{});
+  if (m <= 10) return f(std::integral_constant<int, 10>{});
+  if (m <= 12) return f(std::integral_constant<int, 12>{});
+  if (m <= 16) return f(std::integral_constant<int, 16>{});
+  if (m <= 20) return f(std::integral_constant<int, 20>{});
+  if (m <= 24) return f(std::integral_constant<int, 24>{});
+  if (m <= 32) return f(std::integral_constant<int, 32>{});
+  if (m <= 40) return f(std::integral_constant<int, 40>{});
+  if (m <= 50) return f(std::integral_constant<int, 50>{});
+  return f(std::integral_constant<int, 64>{});
 }
 
 // Position of the (r+1)-th set bit of x (r = 0 for the lowest), r < popc(x):
