@@ -263,7 +263,7 @@ cudaError_t launch_bad_fill(float *cube, long long T, int n, const uint8_t *map,
 cudaError_t launch_bad_pass(const float *src, float *dst, uint32_t D, int n, const uint32_t *frames,
                             unsigned long long *counts, cudaStream_t st);
 
-// register.cu: registration (Sect. 3.1), one CTA per frame
+// register.cu: registration (Sect. 3.1)
 struct RegArgs {
   const float *in;   // T x n x n device
   double *out;       // T x 8 device: found, x0, y0, fwhm, I0, alpha, beta, Bg

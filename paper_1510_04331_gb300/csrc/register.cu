@@ -10,7 +10,7 @@
 //    packed (total-order key of the value, ~index): the largest value wins,
 //    the smallest index on a tie.  A non-finite value sets the word to all
 //    ones (no finite value packs to it) and the status flag.
-//  * register_fit_kernel: one block of FIT_WARPS warps per frame.  The box of
+//  * register_fit_kernel: one block of four or two warps per frame.  The box of
 //    half-size R around the seed and its 8-connected flood fill in shared
 //    memory (sweeps until none changes: the fixpoint is the connected
 //    component whatever the order of the updates), FP64 patch sums, then the
@@ -18,15 +18,16 @@
 //    Warp 0 holds the parameters, solves the damped 6 x 6 system and takes
 //    the decisions; the model and its derivatives are evaluated by every
 //    warp, a pixel per thread, into shared memory, and the 28 sums of the
-//    normal equations are then taken seven to a warp.  Each sum is taken in
-//    one fixed order (32 strided partials, then a butterfly over them).
-//    Start values, damping schedule and stopping rules are those of the FP64
-//    oracle.
-//    Bound: the FP64 pipe (a warp instruction takes it 16 cycles; 14,500 of
-//    them per fitted frame) and, below a few frames per SM, the latency of
-//    the chain evaluate - sum - solve.  With a frame on one warp that chain
-//    was all there was; measured calls, then -> now, same bits: one frame
-//    612 -> 315 us, 400 of 256 x 256 1259 -> 774, 1600 2084 -> 1849.
+//    normal equations are then taken in four groups of seven.  Each sum is
+//    taken in one fixed order (32 strided partials, then a butterfly over
+//    them).  Start values, damping schedule and stopping rules are those of the
+//    FP64 oracle.
+//    Bound: the FP64 pipe (a warp instruction takes it 16 cycles; 14 000 of
+//    them per fitted frame of the 256 x 256 workload) and, below a few frames
+//    per SM, the latency of the chain evaluate - sum - solve.  With a frame on
+//    one warp that chain was all there was; calls with one warp and with four,
+//    same bits: one frame 612 and 315 us, 400 of 256 x 256 1259 and 774, 1600
+//    2084 and 1849.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -39,10 +40,11 @@ namespace {
 constexpr int ARG_THREADS = 256;
 constexpr int ARG_VEC = 8;                                   // float4 loads per thread per chunk
 constexpr long long REG_CHUNK = (long long)ARG_THREADS * ARG_VEC * 4;   // pixels per block
-// Warps per block (frame): the sums take four.  With three blocks per SM 400
-// frames take 779 us; two 887, one 1118, four 781, two of eight warps 872.
-constexpr int FIT_WARPS = 4;
-constexpr int FIT_THREADS = 32 * FIT_WARPS;
+// Twelve warps an SM (register budget), as blocks of WARPS = 4 or 2, a frame
+// each (launch_register_fit chooses).  The bits do not depend on it: warp w
+// takes the groups w, w + WARPS, ... of the sums, each in its one order.
+constexpr int FIT_SM_WARPS = 12;
+constexpr int GROUPS = 4;
 constexpr int FIT_TILE = 512;  // window pixels whose model values are in shared memory at a time
 constexpr int FIT_Z = 6;       // values per pixel there: dI/dI0, dx0, dy0, dalpha, dbeta and the residual
 constexpr double REG_PI = 3.14159265358979323846;
@@ -233,7 +235,11 @@ enum { EVAL_DONE = 0, EVAL_F32 = 1, EVAL_F64 = 2 };
 
 // Barrier of all the block's warps, for the places where warp 0 and the
 // others wait at different instructions.
-__device__ __forceinline__ void fit_sync() { asm volatile("bar.sync 1, %0;" ::"n"(FIT_THREADS) : "memory"); }
+template <int WARPS>
+__device__ __forceinline__ void fit_sync() {
+  if constexpr (WARPS == 1) __syncwarp();
+  else asm volatile("bar.sync 1, %0;" ::"n"(32 * WARPS) : "memory");
+}
 
 // Model values of one pixel at the parameters k: derivatives by I0, x0, y0,
 // alpha, beta (the one by Bg is 1) and the residual.  Where a sum of two
@@ -361,46 +367,47 @@ __device__ __forceinline__ void group_finish(R (&acc)[8], int lane, double *ne) 
 // takes the two in separate passes; one pass serves both here because the
 // normal equations of an accepted trial point are those of the next
 // iteration.
-template <class R, class K>
+template <int WARPS, class R, class K>
 __device__ __forceinline__ void window_pass(const K &k, FitShared &s, R *z, const float *win, int WH, int WW, int wr0,
                                             int wc0) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int np = WH * WW;
-  R acc[8] = {};
+  R acc[GROUPS / WARPS][8] = {};
   for (int t0 = 0; t0 < np; t0 += FIT_TILE) {
     const int count = min(FIT_TILE, np - t0);
-    if (t0 > 0) fit_sync();   // the sums have read the tile before
-    for (int i = threadIdx.x; i < count; i += FIT_THREADS) {
+    if (t0 > 0) fit_sync<WARPS>();   // the sums have read the tile before
+    for (int i = threadIdx.x; i < count; i += 32 * WARPS) {
       const int r = (t0 + i) / WW, c = t0 + i - r * WW;
       R v[FIT_Z];
       moffat_pixel(k, c + wc0, r + wr0, win[t0 + i], v);
 #pragma unroll
       for (int q = 0; q < FIT_Z; q++) z[q * FIT_TILE + i] = v[q];
     }
-    fit_sync();
-    if (wid == 0) group_sums<0>(z, count, lane, acc);
-    else if (wid == 1) group_sums<1>(z, count, lane, acc);
-    else if (wid == 2) group_sums<2>(z, count, lane, acc);
-    else if (wid == 3) group_sums<3>(z, count, lane, acc);
+    fit_sync<WARPS>();
+    if (wid == 0 % WARPS) group_sums<0>(z, count, lane, acc[0 / WARPS]);
+    if (wid == 1 % WARPS) group_sums<1>(z, count, lane, acc[1 / WARPS]);
+    if (wid == 2 % WARPS) group_sums<2>(z, count, lane, acc[2 / WARPS]);
+    if (wid == 3 % WARPS) group_sums<3>(z, count, lane, acc[3 / WARPS]);
   }
-  if (wid == 0) group_finish<0>(acc, lane, s.ne);
-  else if (wid == 1) group_finish<1>(acc, lane, s.ne);
-  else if (wid == 2) group_finish<2>(acc, lane, s.ne);
-  else if (wid == 3) group_finish<3>(acc, lane, s.ne);
-  fit_sync();
+  if (wid == 0 % WARPS) group_finish<0>(acc[0 / WARPS], lane, s.ne);
+  if (wid == 1 % WARPS) group_finish<1>(acc[1 / WARPS], lane, s.ne);
+  if (wid == 2 % WARPS) group_finish<2>(acc[2 / WARPS], lane, s.ne);
+  if (wid == 3 % WARPS) group_finish<3>(acc[3 / WARPS], lane, s.ne);
+  fit_sync<WARPS>();
 }
 
 // The parameters' quotients from shared memory, then the pass.
+template <int WARPS>
 __device__ __forceinline__ void window_pass_shared(int mode, FitShared &s, unsigned char *zb, const float *win, int WH,
                                                    int WW, int wr0, int wc0) {
   if (mode == EVAL_F32) {
     const MoffatConst32 k = {s.kf[0], s.kf[1], s.kf[2], s.kf[3], s.kf[4], s.kf[5],
                              s.kf[6], s.kf[7], s.kf[8], s.kf[9], s.kf[10]};
-    window_pass<float>(k, s, reinterpret_cast<float *>(zb), win, WH, WW, wr0, wc0);
+    window_pass<WARPS, float>(k, s, reinterpret_cast<float *>(zb), win, WH, WW, wr0, wc0);
   } else {
     const MoffatConst k = {s.kc[0], s.kc[1], s.kc[2], s.kc[3], s.kc[4], s.kc[5],
                            s.kc[6], s.kc[7], s.kc[8], s.kc[9], s.kc[10]};
-    window_pass<double>(k, s, reinterpret_cast<double *>(zb), win, WH, WW, wr0, wc0);
+    window_pass<WARPS, double>(k, s, reinterpret_cast<double *>(zb), win, WH, WW, wr0, wc0);
   }
 }
 
@@ -458,7 +465,7 @@ __device__ bool step32(const double *ne, double lambda, double *d) {
 // Evaluation at the parameters p, called by warp 0: hands the quotients to
 // the block and takes part in the pass.  Returns the squared error (the other
 // sums are in s.ne).
-template <bool F32>
+template <int WARPS, bool F32>
 __device__ __forceinline__ double evaluate(const double *p, FitShared &s, unsigned char *zb, const float *win, int WH,
                                            int WW, int wr0, int wc0) {
   const int lane = threadIdx.x & 31;
@@ -473,8 +480,8 @@ __device__ __forceinline__ double evaluate(const double *p, FitShared &s, unsign
     }
     s.mode = F32 ? EVAL_F32 : EVAL_F64;
   }
-  fit_sync();
-  window_pass_shared(F32 ? EVAL_F32 : EVAL_F64, s, zb, win, WH, WW, wr0, wc0);
+  fit_sync<WARPS>();
+  window_pass_shared<WARPS>(F32 ? EVAL_F32 : EVAL_F64, s, zb, win, WH, WW, wr0, wc0);
   return s.ne[27];
 }
 
@@ -484,12 +491,12 @@ __device__ __forceinline__ double evaluate(const double *p, FitShared &s, unsign
 // stop when an accepted step lowers the squared error by at most stop_rel
 // of it, when no try lowers it, or after 200 iterations).  F32 selects the
 // FP32 evaluation.  Returns the iterations made; p and cost are updated.
-template <bool F32>
+template <int WARPS, bool F32>
 __device__ __forceinline__ int lm_loop(double (&p)[6], double &cost, double lam_floor, double stop_rel, FitShared &s,
                                        unsigned char *zb, const float *buf, int WH, int WW, int wr0, int wc0) {
   const int lane = threadIdx.x & 31;
   const double *ne_cur = s.ne_cur;
-  cost = evaluate<F32>(p, s, zb, buf, WH, WW, wr0, wc0);
+  cost = evaluate<WARPS, F32>(p, s, zb, buf, WH, WW, wr0, wc0);
   // the normal equations at p
   if (lane < 27) s.ne_cur[lane] = s.ne[lane];
   __syncwarp();
@@ -532,7 +539,7 @@ __device__ __forceinline__ int lm_loop(double (&p)[6], double &cost, double lam_
         lambda *= 10.0;
         continue;
       }
-      newcost = evaluate<F32>(q, s, zb, buf, WH, WW, wr0, wc0);
+      newcost = evaluate<WARPS, F32>(q, s, zb, buf, WH, WW, wr0, wc0);
       if (newcost < cost) {
 #pragma unroll
         for (int ii = 0; ii < 6; ii++) p[ii] = q[ii];
@@ -559,8 +566,10 @@ __device__ __forceinline__ int lm_loop(double (&p)[6], double &cost, double lam_
 // One frame on one block: seed from the argmax word, patch, centroid, fit.
 // buf: side^2 floats (the box, then the window); lab: side^2 bytes (the
 // patch), the same memory as the model values zb, which come after it.
+template <int WARPS>
 __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long key, long long f, float *buf,
                                           uint8_t *lab, unsigned char *zb, FitShared &s) {
+  constexpr int THREADS = 32 * WARPS;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int n = a.n;
   const float *fr = a.in + f * (long long)n * n;
@@ -587,7 +596,7 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
   // ---- patch: flood fill of the pixels above the threshold ----------------
   // lab: 0 below the threshold, 2 above and not (yet) reached, 1 in the patch
   const int si = (r0 - rlo) * W + (c0 - clo);
-  for (int i = tid; i < H * W; i += FIT_THREADS) {
+  for (int i = tid; i < H * W; i += THREADS) {
     const int r = i / W, c = i - r * W;
     const float v = fr[(long long)(r + rlo) * n + (c + clo)];
     buf[i] = v;
@@ -603,9 +612,9 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
     int changed = 0;
     // 32 pixels a thread at a time: all found against the same labels, then
     // all marked
-    for (int b = 0; b < H * W; b += 32 * FIT_THREADS) {
+    for (int b = 0; b < H * W; b += 32 * THREADS) {
       uint32_t reached = 0;
-      for (int i = b + tid, k = 0; k < 32 && i < H * W; i += FIT_THREADS, k++) {
+      for (int i = b + tid, k = 0; k < 32 && i < H * W; i += THREADS, k++) {
         if (lab[i] != 2) continue;
         const int r = i / W, c = i - r * W;
         bool nb = false;
@@ -618,30 +627,30 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
       }
       __syncthreads();
       changed |= reached != 0;
-      for (; reached; reached &= reached - 1) lab[b + tid + (__ffs(reached) - 1) * FIT_THREADS] = 1;
+      for (; reached; reached &= reached - 1) lab[b + tid + (__ffs(reached) - 1) * THREADS] = 1;
       __syncthreads();
     }
     if (!__syncthreads_or(changed)) break;
   }
-  // the four sums, one to a warp (each in the order of 32 strided partials)
-  if (wid < 4) {
+  // the four sums, warp by warp (each in the order of 32 strided partials)
+  for (int k = wid; k < 4; k += WARPS) {
     double acc = 0.0;
     bool touch = false;
     for (int i = lane; i < H * W; i += 32) {
       if (lab[i] != 1) continue;
       const int r = i / W, c = i - r * W;
       const double v = buf[i];
-      if (wid == 0) {
+      if (k == 0) {
         acc += 1.0;
         touch |= (r == 0 && rlo > 0) || (r == H - 1 && rhi < n - 1) || (c == 0 && clo > 0) || (c == W - 1 && chi < n - 1);
-      } else if (wid == 1) {
+      } else if (k == 1) {
         acc += v;
       } else {
-        acc += v * (double)(wid == 2 ? c + clo : r + rlo);
+        acc += v * (double)(k == 2 ? c + clo : r + rlo);
       }
     }
     acc = warp_sum(acc);
-    if (lane == 0) s.patch[wid] = acc;
+    if (lane == 0) s.patch[k] = acc;
     if (touch) s.touch = 1;
   }
   __syncthreads();
@@ -661,17 +670,17 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
   const int wr0 = max(rc - w, 0), wr1 = min(rc + w, n - 1), wc0 = max(cc - w, 0), wc1 = min(cc + w, n - 1);
   const int WH = max(wr1 - wr0 + 1, 0), WW = max(wc1 - wc0 + 1, 0);
   // the box reads are done: the buffer now takes the window
-  for (int i = tid; i < WH * WW; i += FIT_THREADS) {
+  for (int i = tid; i < WH * WW; i += THREADS) {
     const int r = i / WW, c = i - r * WW;
     buf[i] = fr[(long long)(r + wr0) * n + (c + wc0)];
   }
   __syncthreads();
   if (wid > 0) {   // evaluate what warp 0 asks for
     for (;;) {
-      fit_sync();
+      fit_sync<WARPS>();
       const int mode = s.mode;
       if (mode == EVAL_DONE) return;
-      window_pass_shared(mode, s, zb, buf, WH, WW, wr0, wc0);
+      window_pass_shared<WARPS>(mode, s, zb, buf, WH, WW, wr0, wc0);
     }
   }
   float lmin = INFINITY;
@@ -687,8 +696,8 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
   // system well away from the FP32 noise of J^T J).  Phase B: the FP64
   // iteration of the oracle from there, which converges in a few steps to
   // the same minimum.
-  const int it_a = lm_loop<true>(p, cost, 1e-6, 1e-7, s, zb, buf, WH, WW, wr0, wc0);
-  const int it_b = lm_loop<false>(p, cost, 1e-12, 1e-14, s, zb, buf, WH, WW, wr0, wc0);
+  const int it_a = lm_loop<WARPS, true>(p, cost, 1e-6, 1e-7, s, zb, buf, WH, WW, wr0, wc0);
+  const int it_b = lm_loop<WARPS, false>(p, cost, 1e-12, 1e-14, s, zb, buf, WH, WW, wr0, wc0);
   const int it = it_a + it_b;
   if (lane == 0) {
     s.mode = EVAL_DONE;
@@ -702,7 +711,7 @@ __device__ __forceinline__ void fit_frame(const RegArgs &a, unsigned long long k
     out[7] = p[5];
     if (a.iters) a.iters[f] = it;
   }
-  fit_sync();
+  fit_sync<WARPS>();
 }
 
 // Shared memory of a block: side^2 floats, then the labels or the model values.
@@ -714,9 +723,9 @@ __host__ __device__ inline size_t fit_smem_bytes(int side) {
 
 // Persistent blocks: each takes the next frame from the counter after the
 // per-frame words (no waiting on other blocks).
-__global__ void __launch_bounds__(FIT_THREADS, 3) register_fit_kernel(const RegArgs a,
-                                                                      unsigned long long *__restrict__ keys,
-                                                                      int side) {
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, FIT_SM_WARPS / WARPS)
+register_fit_kernel(const RegArgs a, unsigned long long *__restrict__ keys, int side) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ FitShared s;
   float *buf = reinterpret_cast<float *>(smem);
@@ -728,8 +737,23 @@ __global__ void __launch_bounds__(FIT_THREADS, 3) register_fit_kernel(const RegA
     __syncthreads();
     const long long f = s.frame;
     if (f >= a.T) break;
-    fit_frame(a, keys[f], f, buf, zb, zb, s);
+    fit_frame<WARPS>(a, keys[f], f, buf, zb, zb, s);
   }
+}
+
+template <int WARPS>
+cudaError_t launch_fit(const RegArgs &a, unsigned long long *keys, int sms, cudaStream_t st) {
+  const int side = 2 * (a.R > a.w ? a.R : a.w) + 1;
+  const size_t smem = fit_smem_bytes(side);
+  auto kernel = register_fit_kernel<WARPS>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * WARPS, smem)) != cudaSuccess) return e;
+  long long grid = (long long)(per_sm > 0 ? per_sm : 1) * sms;
+  if (grid > a.T) grid = a.T;
+  kernel<<<(unsigned)grid, 32 * WARPS, smem, st>>>(a, keys, side);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -750,20 +774,21 @@ cudaError_t launch_register_argmax(const RegArgs &a, unsigned long long *keys, c
 
 cudaError_t launch_register_fit(const RegArgs &a, unsigned long long *keys, cudaStream_t st) {
   if (a.T <= 0) return cudaSuccess;
-  const int side = 2 * (a.R > a.w ? a.R : a.w) + 1;
-  const size_t smem = fit_smem_bytes(side);
-  cudaError_t e = cudaFuncSetAttribute(register_fit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0, dev = 0, sms = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, register_fit_kernel, FIT_THREADS, smem)) !=
-      cudaSuccess)
-    return e;
+  int dev = 0, sms = 0;
+  cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  long long grid = (long long)(per_sm > 0 ? per_sm : 1) * sms;
-  if (grid > a.T) grid = a.T;
-  register_fit_kernel<<<(unsigned)grid, FIT_THREADS, smem, st>>>(a, keys, side);
-  return cudaGetLastError();
+  // four warps a frame while all frames are resident at once, and for windows
+  // of more than one tile; else, where the solves on one warp are much of the
+  // work, two, so that twice as many frames are solved at a time.  Calls on
+  // 100 x 100 frames, one / two / four warps a frame and the one-warp fit
+  // without shared sums: w = 4, 300 frames 1251 / 1054 / 954 and 1400 us, 600
+  // 1295 / 1158 / 1550 and 1454, 4000 4558 / 4768 / 6255 and 4988; w = 10, 600
+  // 1335 / 950 / 977 and 1308, 4000 3785 / 3552 / 3799 and 3803; w = 14, 600 2174
+  // / 1510 / 1485 and 2076, 1800 3666 / 3065 / 2979 and 3424.
+  const long long pixels = (2ll * a.w + 1) * (2 * a.w + 1);
+  if (a.T <= (long long)(FIT_SM_WARPS / 4) * sms || pixels > FIT_TILE) return launch_fit<4>(a, keys, sms, st);
+  return launch_fit<2>(a, keys, sms, st);
 }
 
 }  // namespace graphic
