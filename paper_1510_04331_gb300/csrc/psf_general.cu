@@ -657,10 +657,15 @@ cudaError_t launch_adi_general(const AdiArgs &a, cudaStream_t st, int &nl) {
   g.table_bytes = unit_bytes(T);
   const int per = (int)std::min<size_t>((size_t)a.n_units, a.band_scratch_cap / g.table_bytes);
   if (per < 1) return cudaErrorInvalidValue;
-  // 1024 counters from 257 frames on (256: a bin holds all of T <= 256
-  // frames' ties without the radix sort)
-  void (*rank)(GeneralArgs) = T <= 256 ? full_rank_kernel<256> : full_rank_kernel<1024>;
-  const size_t rsmem = SEG * (T <= 256 ? full_pixel_bytes<256>(T) : full_pixel_bytes<1024>(T));
+  // counters: 1024 from 257 frames on, 512 from 129 (512 and 256 alike on plain
+  // noise; one bright frame, which leaves all others in one bin: ranking 256
+  // frames of 512 x 512 4392 us with 256 counters, without the radix sort, 2018
+  // with 512 and the sort, 130 frames 1542 and 1136), 256 below (64 frames 246
+  // us, 265 with 512; one bright frame 456 and 695)
+  void (*rank)(GeneralArgs) = T <= 128 ? full_rank_kernel<256> : T <= 256 ? full_rank_kernel<512> : full_rank_kernel<1024>;
+  const size_t rsmem = SEG * (T <= 128   ? full_pixel_bytes<256>(T)
+                              : T <= 256 ? full_pixel_bytes<512>(T)
+                                         : full_pixel_bytes<1024>(T));
   if (rsmem > kPlainSmem &&
       (e = cudaFuncSetAttribute(rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem)) != cudaSuccess)
     return e;
