@@ -49,20 +49,29 @@ constexpr int C2_KS = 4;
 // 1/64 of its FP32 one: the FP64 test of every value was most of the master
 // sky's time (290 us for 50 frames of 512 x 512, 262144 x 50 x 4 FP64
 // operations at about 2 per SM and cycle being 90 us of it).
-__device__ __forceinline__ bool mask_covers(const CollapseArgs &a, long long t, const float4 f, int col, int row) {
+__device__ __forceinline__ bool mask_filter(const float4 f, int col, int row, float r2, bool &sure) {
   const float dx = (float)col - f.x, dy = (float)row - f.y;
-  const float d2 = fmaf(dx, dx, dy * dy), r2 = (float)a.mask_r2;
+  const float d2 = fmaf(dx, dx, dy * dy);
   const float tol = f.z * (fabsf(dx) + fabsf(dy) + 1.0f) + 4.8e-7f * (d2 + r2);
-  if (fabsf(d2 - r2) > tol) return d2 < r2;
+  sure = fabsf(d2 - r2) > tol;
+  return d2 < r2;
+}
+__device__ __forceinline__ bool mask_exact(const CollapseArgs &a, long long t, int col, int row) {
   const double ex = (double)col - a.mask_x[t], ey = (double)row - a.mask_y[t];
   return ex * ex + ey * ey < a.mask_r2;
+}
+__device__ __forceinline__ bool mask_covers(const CollapseArgs &a, long long t, const float4 f, int col, int row) {
+  bool sure;
+  const bool in = mask_filter(f, col, row, (float)a.mask_r2, sure);
+  return sure ? in : mask_exact(a, t, col, row);
 }
 
 // MASKED (master sky, Sect. 3.2): values that are not finite or fall in the
 // frame's star mask are left out -- they get the largest key, so they rank
 // after every value kept -- and the median is taken over the m values kept
-// (NaN when m = 0).
-template <bool SMEM, bool MASKED = false>
+// (NaN when m = 0).  STARS: there are star masks (the test compiled in but not
+// used: 300 frames of 512 x 512 452 us instead of 423).
+template <bool SMEM, bool MASKED = false, bool STARS = false>
 __global__ void __launch_bounds__(32 * COL_PPC) collapse_kernel(const CollapseArgs a) {
   extern __shared__ uint32_t csm[];
   uint32_t *hist_all = csm;                       // [COL_PPC][256]
@@ -84,12 +93,13 @@ __global__ void __launch_bounds__(32 * COL_PPC) collapse_kernel(const CollapseAr
   }
   uint32_t *hist = hist_all + w * 256;
   const long long p = p0 + w;
+  const int row = (int)((unsigned)p / (unsigned)a.n), col = (int)((unsigned)p - (unsigned)row * (unsigned)a.n);
   // masked-out values (MASKED) get the largest key
   auto key_of = [&](long long t, float v) -> uint32_t {
     if constexpr (MASKED) {
       bool keep = isfinite(v);
-      if (a.mask_x) {
-        keep &= !mask_covers(a, t, __ldg(&a.maskf[t]), (int)(p % a.n), (int)(p / a.n));
+      if constexpr (STARS) {
+        if (a.mask_x) keep &= !mask_covers(a, t, __ldg(&a.maskf[t]), (int)(p % a.n), (int)(p / a.n));
       }
       return keep ? f2key(v) : 0xffffffffu;
     } else {
@@ -104,16 +114,50 @@ __global__ void __launch_bounds__(32 * COL_PPC) collapse_kernel(const CollapseAr
   // digits shared by every key
   uint32_t orv = 0, andv = 0xffffffffu;
   int kept = 0;
-  for (long long t = lane; t < T; t += 32) {
-    float v;
-    if constexpr (SMEM) v = __uint_as_float(keys_all[t * COL_KS + w]);
-    else v = a.in[t * NN + p];
-    const uint32_t key = key_of(t, v);
-    if constexpr (MASKED) kept += (key != 0xffffffffu) ? 1 : 0;
-    else bad |= !isfinite(v);
-    if constexpr (SMEM) keys_all[t * COL_KS + w] = key;
-    orv |= key;
-    andv &= key;
+  if constexpr (SMEM && STARS) {
+    // four frames a step: their masks are loaded together, and the FP64 test at
+    // a rim is out of the way (300 frames of 512 x 512 622 us; a frame at a time
+    // 670, FP64 tests only 978)
+    const float r2 = (float)a.mask_r2;
+    for (long long t0 = lane; t0 - lane < T; t0 += 128) {
+      bool in[4], sure[4], all = true;
+      float4 f[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) f[u] = __ldg(&a.maskf[t0 + 32 * u < T ? t0 + 32 * u : T - 1]);
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        in[u] = mask_filter(f[u], col, row, r2, sure[u]);
+        all &= sure[u] || t0 + 32 * u >= T;
+      }
+      if (!all) {
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+          if (!sure[u] && t0 + 32 * u < T) in[u] = mask_exact(a, t0 + 32 * u, col, row);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        if (t0 + 32 * u >= T) continue;
+        uint32_t *at = &keys_all[(t0 + 32 * u) * COL_KS + w];
+        const float v = __uint_as_float(*at);
+        const uint32_t key = isfinite(v) && !in[u] ? f2key(v) : 0xffffffffu;
+        kept += key != 0xffffffffu ? 1 : 0;
+        *at = key;
+        orv |= key;
+        andv &= key;
+      }
+    }
+  } else {
+    for (long long t = lane; t < T; t += 32) {
+      float v;
+      if constexpr (SMEM) v = __uint_as_float(keys_all[t * COL_KS + w]);
+      else v = a.in[t * NN + p];
+      const uint32_t key = key_of(t, v);
+      if constexpr (MASKED) kept += (key != 0xffffffffu) ? 1 : 0;
+      else bad |= !isfinite(v);
+      if constexpr (SMEM) keys_all[t * COL_KS + w] = key;
+      orv |= key;
+      andv &= key;
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -496,13 +540,14 @@ cudaError_t launch_sky_median(const CollapseArgs &a, cudaStream_t st) {
   const unsigned grid = (unsigned)(NN / COL_PPC);
   if (a.T <= 8192) {
     const size_t smem = (size_t)(COL_PPC * 256 + COL_KS * a.T) * sizeof(uint32_t);
-    cudaError_t e = cudaFuncSetAttribute(collapse_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    void (*const kernel)(CollapseArgs) = a.mask_x ? collapse_kernel<true, true, true> : collapse_kernel<true, true>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    collapse_kernel<true, true><<<grid, 32 * COL_PPC, smem, st>>>(a);
+    kernel<<<grid, 32 * COL_PPC, smem, st>>>(a);
   } else {
     const size_t smem = (size_t)(COL_PPC * 256) * sizeof(uint32_t);
-    collapse_kernel<false, true><<<grid, 32 * COL_PPC, smem, st>>>(a);
+    if (a.mask_x) collapse_kernel<false, true, true><<<grid, 32 * COL_PPC, smem, st>>>(a);
+    else collapse_kernel<false, true><<<grid, 32 * COL_PPC, smem, st>>>(a);
   }
   return cudaGetLastError();
 }
