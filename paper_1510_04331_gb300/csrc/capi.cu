@@ -37,7 +37,7 @@ struct graphic_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   int *d_status = nullptr;
-  int *h_status = nullptr;          // pinned: the status word, then from word 2 on 16 bytes of results read back by a call
+  int *h_status = nullptr;          // pinned: the status word; 16 bytes of results read back from word 2 on
   char *d_plan = nullptr;
   size_t d_plan_bytes = 0;
   char *h_plan = nullptr;           // pinned staging
@@ -278,11 +278,8 @@ int graphic::validate_shift(const double *dx, const double *dy, int64_t T, int32
 
 namespace {
 
-// Enqueue the two shift passes for frames [0, T) with parameters at device
-// pointers p_dx, p_dy.  in -> out (out may equal in); in_fs / out_fs: the
-// frame strides in elements (0: n*n).
-// The per-frame shift parameters of both passes for T frames, the x table
-// then the y table, to c->d_lparam.
+// The per-frame shift parameters of both passes for T frames, from device
+// pointers p_dx, p_dy: the x table, then the y table, to c->d_lparam.
 int shift_params(graphic_ctx *c, int64_t T, int32_t n, const double *p_dx, const double *p_dy) {
   const size_t pb = line_params_bytes(SHIFT_X, n, T);
   int rc = ensure(c, (void **)&c->d_lparam, &c->lparam_bytes, 2 * pb, false);
@@ -295,7 +292,8 @@ int shift_params(graphic_ctx *c, int64_t T, int32_t n, const double *p_dx, const
   return e == cudaSuccess ? GRAPHIC_OK : cuda_fail(e, "shift parameters");
 }
 
-// Both passes of frames [f0, f1) of the T that shift_params was called for.
+// Both passes of frames [f0, f1) of the T that shift_params was called for,
+// in -> out (out may equal in); in_fs / out_fs: the frame strides in elements.
 int shift_passes(graphic_ctx *c, const float *in, float *out, int64_t T, int64_t f0, int64_t f1, int32_t n,
                  const double *p_dx, const double *p_dy, long long in_fs, long long out_fs) {
   const size_t pb = line_params_bytes(SHIFT_X, n, T);
@@ -328,6 +326,7 @@ int shift_passes(graphic_ctx *c, const float *in, float *out, int64_t T, int64_t
   return GRAPHIC_OK;
 }
 
+// Parameters and both passes of all T frames (frame strides 0: n*n).
 int enqueue_shift(graphic_ctx *c, const float *in, float *out, int64_t T, int32_t n, const double *p_dx,
                   const double *p_dy, long long in_fs = 0, long long out_fs = 0) {
   const long long NN = (long long)n * n;

@@ -24,11 +24,11 @@
 //     keeps the number of members below its pointer, and moves the pointer by
 //     the few set bits that the median moved.  Values in and residuals out
 //     move as whole sectors.
-// Before (one kernel, 8 pixels per CTA and one CTA per SM: a radix sort per
-// pixel, then queries across the lanes, each lane meeting its events at other
-// queries and walking its own words): 600 frames of 256 x 256 with a time
-// gate 3.61 ms, so 1.21 (ranking 0.48, sweep 0.73); 2000 frames of 128 x 128
-// 2.86 ms.  Bound by instruction issue (65 %) and the codes' loads.
+// Against one kernel with 8 pixels per CTA and one CTA per SM (a radix sort
+// per pixel, then queries across the lanes, each lane meeting its events at
+// other queries and walking its own words): 600 frames of 256 x 256 with a
+// time gate 3.61 ms, so 1.14 (ranking 0.46, sweep 0.68).  Bound by instruction
+// issue (65 %) and the codes' loads.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

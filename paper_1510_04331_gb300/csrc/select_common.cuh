@@ -30,7 +30,8 @@ __device__ __forceinline__ float key2f(uint32_t k) {
 // the a with edge2[a] <= rho^2 < edge2[a + 1] for whole squared radii, the
 // edges in increasing order.  In 32-bit integers: the same comparisons in FP64
 // took the narrow FP64 pipe 16 cycles each and kept it busy for 47 % of
-// band_prep_kernel on 32 frames of 512 x 512 (384 us, 339 now).
+// band_prep_kernel on 32 frames of 512 x 512 (384 us, 339 with integers and all
+// else as it was).
 __device__ __forceinline__ int annulus_of(long long pixel, int n, const int *__restrict__ iedge2, int n_ann) {
   const unsigned p = (unsigned)pixel, row = p / (unsigned)n;
   const int x = (int)(p - row * (unsigned)n) - n / 2, y = (int)row - n / 2;
