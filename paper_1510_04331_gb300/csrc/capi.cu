@@ -235,8 +235,9 @@ int end_call(graphic_ctx *c) {
 
 // Frames of one host -> device copy piece of graphic_reduce_host: an eighth of
 // the cube, so that only the last eighth's shift is left when the copy ends
-// (250 x 512 x 512: 4128 us, in one piece of 256 MiB 4427), from 16 MiB (two
-// passes over it still fill the chip) to 256 MiB (an eighth of a survey cube).
+// (250 x 512 x 512: 3892 us, in one piece of 256 MiB 4201; 60 x 512 x 512 1262
+// and 1328, 1000 x 512 x 512 14 306 and 14 443), from 16 MiB (two passes over it
+// still fill the chip) to 256 MiB (an eighth of a survey cube).
 long long copy_piece_frames(long long T, size_t bytes_per_frame) {
   const size_t eighth = (size_t)T * bytes_per_frame / 8;
   const size_t piece = std::min<size_t>(std::max<size_t>(eighth, (size_t)16 << 20), (size_t)256 << 20);

@@ -30,8 +30,6 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <type_traits>
-
 #include "graphic_internal.h"
 #include "line_common.cuh"
 
@@ -356,7 +354,9 @@ __device__ __forceinline__ void stage_columns(const float *__restrict__ src, siz
   }
 }
 
-template <int M, int KIND, int TH, bool CG = false>
+// ANY: the frames that rotation pass 1 reads may start at any float address
+// (frames_any); no staging, no loads of pairs.
+template <int M, int KIND, int TH, bool CG = false, bool ANY = false>
 __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, int cx, float2 *smem, LineParam *lp,
                                                int *ident_p) {
   constexpr int N = M / 2;
@@ -409,8 +409,7 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
         } else if constexpr (KIND == SHIFT_Y) {
           z = ldf2<CG>(fin + (size_t)pos * N + line0);
         } else if constexpr (KIND == ROT_P1) {
-          z = aligned(fin, 8) ? load_rot90_pair<CG>(fin, N, q, line0, pos)
-                              : load_rot90_pair<CG, false>(fin, N, q, line0, pos);
+          z = load_rot90_pair<CG, !ANY>(fin, N, q, line0, pos);
         }
       }
       if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
@@ -443,7 +442,7 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
   if constexpr (KIND == ROT_P1 && STAGE) {
     // an odd number of quarter turns: the rows of rot90^q(frame) are columns
     // of the frame
-    staged = (q & 1) && aligned(fin, 16);
+    staged = !ANY && (q & 1);
     if (staged) {
       if (q == 1) {   // element pos >= 1 of line i is frame[n - pos][i]; element 0 is zero
         stage_columns<N, LPC, TH, LBUF, CG>(fin + col0, N, stage, [](int row) { return row ? N - row : -1; });
@@ -488,30 +487,26 @@ __device__ __forceinline__ void line_pass_body(const LineArgs &a, long long f, i
       if (bad) atomicOr(a.status, STATUS_NONFINITE);
     }
   } else {
-    auto load = [&](auto pair) {
 #pragma unroll
-      for (int m = 0; m < 16; m++) {
-        const int pos = j + m * (M / 16);
-        float2 z = make_float2(0.f, 0.f);
-        if (m * (M / 16) < NIN) {   // compile-time pruning of the zero half
-          if constexpr (KIND == SHIFT_X) {
-            z = make_float2(ldf<CG>(fin + (size_t)line0 * N + pos), ldf<CG>(fin + (size_t)(line0 + 1) * N + pos));
-          } else if constexpr (KIND == SHIFT_Y) {
-            z = ldf2<CG>(fin + (size_t)pos * N + line0);
-          } else if constexpr (KIND == ROT_P1) {
-            z = load_rot90_pair<CG, decltype(pair)::value>(fin, N, q, line0, pos);
-          } else if constexpr (KIND == ROT_P2) {
-            z = ldf2<CG>(fin + (size_t)pos * M + line0);
-          } else {
-            z = make_float2(ldf<CG>(fin + (size_t)line0 * M + pos), ldf<CG>(fin + (size_t)(line0 + 1) * M + pos));
-          }
-          if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
+    for (int m = 0; m < 16; m++) {
+      const int pos = j + m * (M / 16);
+      float2 z = make_float2(0.f, 0.f);
+      if (m * (M / 16) < NIN) {   // compile-time pruning of the zero half
+        if constexpr (KIND == SHIFT_X) {
+          z = make_float2(ldf<CG>(fin + (size_t)line0 * N + pos), ldf<CG>(fin + (size_t)(line0 + 1) * N + pos));
+        } else if constexpr (KIND == SHIFT_Y) {
+          z = ldf2<CG>(fin + (size_t)pos * N + line0);
+        } else if constexpr (KIND == ROT_P1) {
+          z = load_rot90_pair<CG, !ANY>(fin, N, q, line0, pos);
+        } else if constexpr (KIND == ROT_P2) {
+          z = ldf2<CG>(fin + (size_t)pos * M + line0);
+        } else {
+          z = make_float2(ldf<CG>(fin + (size_t)line0 * M + pos), ldf<CG>(fin + (size_t)(line0 + 1) * M + pos));
         }
-        v[m] = z;
+        if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
       }
-    };
-    if (KIND == ROT_P1 && !aligned(fin, 8)) load(std::false_type{});
-    else load(std::true_type{});
+      v[m] = z;
+    }
     if constexpr (KIND == SHIFT_X || KIND == ROT_P1) {
       if (bad) atomicOr(a.status, STATUS_NONFINITE);
     }
@@ -625,13 +620,13 @@ constexpr int line_threads() { return (M == 2048 && (KIND == SHIFT_Y || KIND == 
 // Register budget: 24 resident warps per SM for lines of up to 256 points, 16
 // for longer ones (measured: 24 is faster on the short lines, slower on the
 // 2048-point ones).
-template <int M, int KIND>
+template <int M, int KIND, bool ANY = false>
 __global__ void __launch_bounds__(line_threads<M, KIND>(), ((M <= 256) ? 768 : 512) / line_threads<M, KIND>())
 line_pass_kernel(const LineArgs a) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ LineParam lp[2 * line_threads<M, KIND>() * 16 / M];
   __shared__ int ident_s;
-  line_pass_body<M, KIND, line_threads<M, KIND>()>(a, blockIdx.y, blockIdx.x, smem, lp, &ident_s);
+  line_pass_body<M, KIND, line_threads<M, KIND>(), false, ANY>(a, blockIdx.y, blockIdx.x, smem, lp, &ident_s);
 }
 
 // ---------------------------------------------------------------------------
@@ -850,7 +845,7 @@ constexpr int w32_ppc() { return (KIND == ROT_P2 || KIND == ROT_P1) ? 8 : 4; }
 constexpr int w32_buf(int ppc) { return 1024 + 32 + (ppc == 8 ? 2 : 4); }
 constexpr size_t w32_smem_bytes(int ppc) { return (size_t)ppc * w32_buf(ppc) * sizeof(float2); }
 
-template <int KIND>
+template <int KIND, bool ANY = false>
 __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) line_pass_w32(const LineArgs a) {
   constexpr int M = 1024, N = 512, PPC = w32_ppc<KIND>();
   constexpr bool SAME_D = (KIND == SHIFT_X || KIND == SHIFT_Y);
@@ -897,8 +892,7 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
         } else if constexpr (KIND == SHIFT_Y) {
           z = *reinterpret_cast<const float2 *>(fin + (size_t)pos * N + line0);
         } else if constexpr (KIND == ROT_P1) {
-          z = aligned(fin, 8) ? load_rot90_pair(fin, N, q, line0, pos)
-                              : load_rot90_pair<false, false>(fin, N, q, line0, pos);
+          z = load_rot90_pair<false, !ANY>(fin, N, q, line0, pos);
         }
       }
       if constexpr (KIND == SHIFT_X || KIND == ROT_P1) bad |= !finite_pair(z);
@@ -944,7 +938,7 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
   //   q = 1: element pos >= 1 of lines col0 + j is frame[n - pos][col0 + j];
   //   q = 3: element pos of line i >= 1 is frame[pos][n - i], i.e. columns
   //          n - col0 - 7 .. n - col0 for the CTA's lines col0 .. col0 + 7.
-  const bool RCOLS = (KIND == ROT_P1) && (q & 1) && aligned(fin, 16);
+  const bool RCOLS = (KIND == ROT_P1) && !ANY && (q & 1);
   if (RCOLS) {
     if (q == 1) {
       constexpr int IT = HP * N / (32 * PPC);
@@ -1000,8 +994,7 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
     // one branch per line pair, not per element, so that each form's loads
     // are issued together: staged columns (odd quarter turns), rows (q = 0)
     // or rows read backwards (q = 2: element pos >= 1 of line i >= 1 is
-    // frame[n - i][n - pos]); column by column where the frame is not aligned
-    // for staging
+    // frame[n - i][n - pos]); ANY: odd quarter turns element by element
     if (RCOLS) {
 #pragma unroll
       for (int m = 0; m < 32; m++) v[m] = (32 * m < NIN) ? buf[pad32(lane + 32 * m)] : make_float2(0.f, 0.f);
@@ -1012,7 +1005,7 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
         v[m] = (32 * m < NIN) ? make_float2(fin[(size_t)line0 * N + pos], fin[(size_t)(line0 + 1) * N + pos])
                               : make_float2(0.f, 0.f);
       }
-    } else if (q & 1) {
+    } else if (ANY && (q & 1)) {
 #pragma unroll
       for (int m = 0; m < 32; m++)
         v[m] = (32 * m < NIN) ? load_rot90_pair<false, false>(fin, N, q, line0, lane + 32 * m) : make_float2(0.f, 0.f);
@@ -1088,6 +1081,16 @@ __global__ void __launch_bounds__(32 * w32_ppc<KIND>(), 16 / w32_ppc<KIND>()) li
   }
 }
 
+// The frames that rotation pass 1 reads are the caller's.  The allocation-free
+// rotation takes them at any float address (every other frame of the library
+// is 16-byte aligned); the frame stride is a multiple of 16 bytes, so all
+// frames of a launch take the same form.  A kernel of its own for those: with
+// both forms in one the aligned frames' pass 1 took 429 us against 425 (400
+// frames of 512 x 512).
+inline bool frames_any(int kind, const LineArgs &a) {
+  return kind == ROT_P1 && !a.in_tab && ((uintptr_t)a.in & 15) != 0;
+}
+
 template <int KIND>
 cudaError_t launch_w32(const LineArgs &a, long long n_frames, cudaStream_t st) {
   constexpr int M = 1024, N = 512, PPC = w32_ppc<KIND>();
@@ -1104,6 +1107,14 @@ cudaError_t launch_w32(const LineArgs &a, long long n_frames, cudaStream_t st) {
     b.out_tab = a.out_tab ? a.out_tab + f0 : nullptr;
     b.lp_tab = a.lp_tab ? reinterpret_cast<const LineParam *>(a.lp_tab) + f0 * a.lp_lines : nullptr;
     dim3 grid(NLINES / (2 * PPC), (unsigned)nf);
+    if constexpr (KIND == ROT_P1) {
+      if (frames_any(KIND, a)) {
+        line_pass_w32<KIND, true><<<grid, 32 * PPC, w32_smem_bytes(PPC), st>>>(b);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        continue;
+      }
+    }
     line_pass_w32<KIND><<<grid, 32 * PPC, w32_smem_bytes(PPC), st>>>(b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1251,6 +1262,14 @@ cudaError_t launch_one(const LineArgs &a, long long n_frames, cudaStream_t st) {
     b.out_tab = a.out_tab ? a.out_tab + f0 : nullptr;
     b.lp_tab = a.lp_tab ? reinterpret_cast<const LineParam *>(a.lp_tab) + f0 * a.lp_lines : nullptr;
     dim3 grid(NLINES / (2 * LPC), (unsigned)nf);
+    if constexpr (KIND == ROT_P1) {
+      if (frames_any(KIND, a)) {
+        line_pass_kernel<M, KIND, true><<<grid, TH, smem, st>>>(b);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        continue;
+      }
+    }
     line_pass_kernel<M, KIND><<<grid, TH, smem, st>>>(b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1281,6 +1300,7 @@ bool configure_m() {
   return set(line_pass_kernel<M, SHIFT_X>, line_threads<M, SHIFT_X>(), SHIFT_X) &&
          set(line_pass_kernel<M, SHIFT_Y>, line_threads<M, SHIFT_Y>(), SHIFT_Y) &&
          set(line_pass_kernel<M, ROT_P1>, line_threads<M, ROT_P1>(), ROT_P1) &&
+         set(line_pass_kernel<M, ROT_P1, true>, line_threads<M, ROT_P1>(), ROT_P1) &&
          set(line_pass_kernel<M, ROT_P2>, line_threads<M, ROT_P2>(), ROT_P2) &&
          set(line_pass_kernel<M, ROT_P3>, line_threads<M, ROT_P3>(), ROT_P3);
 }
@@ -1336,6 +1356,7 @@ int geom_init_device() {
     if (cudaFuncSetAttribute(line_pass_w32<SHIFT_X>, at, (int)w32_smem_bytes(w32_ppc<SHIFT_X>())) != cudaSuccess ||
         cudaFuncSetAttribute(line_pass_w32<SHIFT_Y>, at, (int)w32_smem_bytes(w32_ppc<SHIFT_Y>())) != cudaSuccess ||
         cudaFuncSetAttribute(line_pass_w32<ROT_P1>, at, (int)w32_smem_bytes(w32_ppc<ROT_P1>())) != cudaSuccess ||
+        cudaFuncSetAttribute(line_pass_w32<ROT_P1, true>, at, (int)w32_smem_bytes(w32_ppc<ROT_P1>())) != cudaSuccess ||
         cudaFuncSetAttribute(line_pass_w32<ROT_P2>, at, (int)w32_smem_bytes(w32_ppc<ROT_P2>())) != cudaSuccess ||
         cudaFuncSetAttribute(line_pass_w32<ROT_P3>, at, (int)w32_smem_bytes(w32_ppc<ROT_P3>())) != cudaSuccess)
       return -1;

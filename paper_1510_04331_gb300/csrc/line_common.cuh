@@ -119,11 +119,5 @@ __device__ __forceinline__ float2 load_rot90_pair(const float *__restrict__ fr, 
   return make_float2(x0, x1);
 }
 
-// The frames of rotation pass 1 are the caller's: the allocation-free
-// rotation takes them at any float address (every other frame of the library
-// is 16-byte aligned, and so are the scratch frames).  The frame stride is a
-// multiple of 16 bytes, so all frames of a launch take the same form.
-__device__ __forceinline__ bool aligned(const float *p, int bytes) { return ((uintptr_t)p & (bytes - 1)) == 0; }
-
 }  // namespace
 }  // namespace graphic
