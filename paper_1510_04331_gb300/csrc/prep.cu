@@ -332,24 +332,24 @@ __global__ void __launch_bounds__(FILL_THREADS) bad_fill_kernel(float *cube, lon
   const long long nn = (long long)n * n;
   const float NANF = __uint_as_float(0x7fc00000u);
   const uint32_t few = list_cap(1, nn);
-  __shared__ uint32_t kept_s, many_s;
+  __shared__ uint32_t kept_s;
   for (long long f = blockIdx.x; f < T; f += gridDim.x) {
     float *fr = cube + f * nn;
     uint32_t *list = lists + f * nn;
     float *vals = reinterpret_cast<float *>(list + cap);   // cap + cap <= nn
     uint32_t left = counts[2 + f];
     if (left > few) {
-      // the frames that would share the dense passes
-      if (threadIdx.x == 0) many_s = 0u;
-      __syncthreads();
-      uint32_t many = 0u;
-      for (long long t = threadIdx.x; t < T; t += FILL_THREADS) many += counts[2 + t] > few ? 1u : 0u;
-      many = __reduce_add_sync(0xffffffffu, many);
-      if ((threadIdx.x & 31) == 0) atomicAdd(&many_s, many);
-      __syncthreads();
-      many = many_s;
-      __syncthreads();
-      if (left > list_cap(many, nn)) {
+      // count the frames that would share the dense passes, from this one on
+      // and only until they allow the list (to the end with at most 160 such
+      // frames: list_cap has then reached half of a frame)
+      bool dense = left > cap;
+      long long many = 0;
+      for (long long i = 0; !dense && left > list_cap(many, nn); i += FILL_THREADS) {
+        const long long t = i + threadIdx.x, u = f + t < T ? f + t : f + t - T;
+        many += __syncthreads_count(t < T && counts[2 + u] > few);
+        dense = i + FILL_THREADS >= T && left > list_cap(many, nn);
+      }
+      if (dense) {
         if (threadIdx.x == 0) counts[2 + T + atomicAdd(&counts[0], 1u)] = (uint32_t)f;
         continue;
       }
