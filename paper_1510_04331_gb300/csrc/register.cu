@@ -778,16 +778,18 @@ cudaError_t launch_register_fit(const RegArgs &a, unsigned long long *keys, cuda
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  // four warps a frame while all frames are resident at once, and for windows
-  // of more than one tile; else, where the solves on one warp are much of the
-  // work, two, so that twice as many frames are solved at a time.  Calls on
-  // 100 x 100 frames, one / two / four warps a frame and the one-warp fit
-  // without shared sums: w = 4, 300 frames 1251 / 1054 / 954 and 1400 us, 600
-  // 1295 / 1158 / 1550 and 1454, 4000 4558 / 4768 / 6255 and 4988; w = 10, 600
-  // 1335 / 950 / 977 and 1308, 4000 3785 / 3552 / 3799 and 3803; w = 14, 600 2174
-  // / 1510 / 1485 and 2076, 1800 3666 / 3065 / 2979 and 3424.
+  // Four warps a frame while about all frames are resident at once, and for
+  // windows of more than one tile; else, where the solves on one warp are much
+  // of the work, two, so that twice as many frames are solved at a time.  The
+  // fewer the pixels, the sooner.  Calls on 100 x 100 frames (a tenth lost), two
+  // and four warps, and one warp without shared sums: w = 4, 480 frames 1112,
+  // 1026, 1430 us, 560 1162, 1434, 1436, 1000 1405, 1849, 1767, 4000 4768, 6255,
+  // 4988; w = 8, 560 819, 778, 1175, 720 923, 975, 1222, 4000 3033, 3387, 3247; w
+  // = 10, 608 949, 966, 1310, 912 1196, 1165, 1473, 1800 1838, 1937, 2139; w = 14,
+  // 720 1708, 1618, 2238, 1800 3065, 2979, 3424.
   const long long pixels = (2ll * a.w + 1) * (2 * a.w + 1);
-  if (a.T <= (long long)(FIT_SM_WARPS / 4) * sms || pixels > FIT_TILE) return launch_fit<4>(a, keys, sms, st);
+  const long long four = pixels <= 128 ? 7ll * sms / 2 : pixels <= 300 ? 4ll * sms : 10ll * sms;
+  if (a.T <= four || pixels > FIT_TILE) return launch_fit<4>(a, keys, sms, st);
   return launch_fit<2>(a, keys, sms, st);
 }
 

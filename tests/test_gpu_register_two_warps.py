@@ -10,12 +10,12 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("R,w", [(6, 3), (8, 5), (16, 10), (32, 8), (32, 11)])
-def test_same_bits_as_short_calls(R, w):
+@pytest.mark.parametrize("R,w,T", [(6, 3, 977), (8, 5, 533), (16, 10, 977), (16, 10, 1611), (32, 8, 977), (32, 11, 977)])
+def test_same_bits_as_short_calls(R, w, T):
     from paper_1510_04331_gb300 import graphic as g
     d = synth.star_frames(70, 96, seed=40 + w, jitter=10.0, fwhm=4.0, lost=0.15)
     few = torch.from_numpy(d.cube).cuda()
-    x = few.repeat(14, 1, 1)[:977].contiguous()
+    x = few.repeat(-(-T // 70), 1, 1)[:T].contiguous()
     args = (0.1 * d.peak, R, 3, 600, w)
     it, it_few = (torch.zeros(len(c), dtype=torch.int32, device="cuda") for c in (x, few))
     got = g.graphic_register(x, *args, iters=it)
